@@ -77,7 +77,7 @@ def bytes_per_cell(kernel: str, f64: bool, phi_frac: float) -> float:
 # x, r out).
 def pcg_schedule_bytes(form: int, f64: bool) -> float:
     S = 8 if f64 else 4
-    return {1: 9 * S, 5: 6 * S + 3 * 0.375 * S}.get(form, 10 * S)
+    return {1: 9 * S, 3: 2 * S + 2 * 0.375 * S, 5: 6 * S + 3 * 0.375 * S}.get(form, 10 * S)
 
 
 PROFILE = "profiles/pcg_sphere_16x8x8_B16_mixed.md"

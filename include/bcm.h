@@ -126,7 +126,8 @@ typedef struct {
     double umax;           /* max |u| after the last step */
     int32_t pcg_form;      /* PCG of the last solve: 0 two launches per iteration,
                               1 persistent streaming, 2 persistent single-reduction,
-                              3 persistent with the state on chip, 4 multigrid-
+                              3 persistent with the state on chip (the default where it
+                              fits), 4 multigrid-
                               preconditioned (two launches and a V-cycle), 5 persistent
                               fused (one grid barrier per iteration, bulk-copy staging) */
     int32_t cn_iters;      /* QUICK + Crank-Nicolson: iterations of the last momentum
@@ -215,7 +216,11 @@ bcm_status bcm_set_solver(bcm_grid *grid, double inner_rtol, int max_cycles, int
 bcm_status bcm_get_solver(const bcm_grid *grid, double *inner_rtol, int32_t *max_cycles,
                           int32_t *check_every, double *barrier_timeout_s, int32_t *recycle);
 
-/* Launch shape of the PCG.  persistent = 5 (mixed mode on 16^3 cubes, grids of at most
+/* Launch shape of the PCG.  Until this call asks for one, a Jacobi solve whose vectors fit
+ * the registers and shared memory of the GPU (grids of at most 256 sims; on 152 SMs of
+ * 227 KB about 4.3M cells in FP32 inner solves and 1.6M in FP64) runs in the on-chip form
+ * (bcm_stats.pcg_form 3), and larger ones persistent = 1 in mixed mode, persistent = 0 in
+ * FP64.  persistent = 5 (mixed mode on 16^3 cubes, grids of at most
  * 160 sims and 256 cubes per SM): one cooperative launch per solve, one block of 1024
  * threads (four x-adjacent cells of the cube in hand each) per SM,
  * one grid barrier per iteration (the beta of the next iteration follows from <q,z> and
@@ -225,10 +230,11 @@ bcm_status bcm_get_solver(const bcm_grid *grid, double *inner_rtol, int32_t *max
  * cooperative launch whose blocks loop over the iterations with two grid-wide barriers
  * each, streaming the vectors through global memory (the mixed-mode default; in a
  * defect-correction cycle it also adds its correction to the FP64 pressure before it
- * returns, where the other forms launch BCM_K_ADD_CORRECTION);
- * persistent = 3: the same iteration with each cube's search direction kept in
- * shared memory, when every cube fits a co-resident block of at most two cubes (FP32
- * inner solve, 16^3 or 8^3 cubes, slabs_a = 1), else the streaming form; persistent = 2:
+ * returns, as form 3 does and where the other forms launch BCM_K_ADD_CORRECTION);
+ * persistent = 3: the same iteration on chip: the preconditioned residual in registers,
+ * the search direction with its ghost planes in shared memory, only the cubes' face values
+ * and the partial sums crossing between blocks (FP32 inner solve that fits, slabs_a = 1),
+ * else the streaming form; persistent = 2:
  * the single-reduction form of the iteration (Chronopoulos-Gear: one pass and one
  * barrier per iteration, three more vectors, the same iterates in exact arithmetic).
  * slabs_a = z-slabs per cube of the streaming work items (1, 2 or 4; 16^3 cubes only
@@ -433,11 +439,11 @@ enum {
     BCM_K_RESIDUAL = 3,       /* FP64 residual (PCG start / defect-correction cycle) */
     BCM_K_CG_A = 4,           /* PCG pass A: new direction, K p, <p, Kp> */
     BCM_K_CG_B = 5,           /* PCG pass B: iterate and residual update, <r,z>, <r,r> */
-    BCM_K_ADD_CORRECTION = 6, /* mixed: x += e (forms other than persistent = 1) */
+    BCM_K_ADD_CORRECTION = 6, /* mixed: x += e (forms other than persistent = 1 and 3) */
     BCM_K_CORRECT = 7,        /* projection + FP64 divergence check */
     BCM_K_MISC = 8,           /* bookkeeping and test-path kernels */
     BCM_K_PCG = 9,            /* persistent PCG: all iterations of one solve (with
-                                 persistent = 1 also the cycle's x += e) */
+                                 persistent = 1 or 3 also the cycle's x += e) */
     BCM_K_MG = 10,            /* multigrid V-cycle (BCM_PRECOND_MULTIGRID) */
     BCM_K_IB = 11,            /* Lagrangian particles: forcing, position update, sets */
     BCM_NKERNELS = 12

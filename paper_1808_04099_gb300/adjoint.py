@@ -48,7 +48,6 @@ class AdjointRun:
         self.rtol = rtol
         self.max_iter = max_iter
         self.g = bcm.Grid(self.spec, bcm.PREC_F64)
-        self.g.set_launch(1, 1, persistent=False)
         self.state0 = state if state is not None else W.initial_state(self.spec)
         L = bcm.lib()
         self.adj_bytes = L.bcm_adjoint_bytes(self.g._h)

@@ -26,6 +26,8 @@ namespace bcm {
 const Ctx* grid_ctx(const bcm_grid* g);
 int grid_two_level(const bcm_grid* g);
 cudaStream_t grid_stream(const bcm_grid* g);
+unsigned long long grid_barrier_timeout_ns(const bcm_grid* g);
+bcm_status grid_read_err(bcm_grid* g);
 bcm_status grid_fail(bcm_status st, const char* msg);
 }  // namespace bcm
 
@@ -514,10 +516,18 @@ extern "C" bcm_status bcm_adjoint_step(bcm_grid* grid, void* dev_adj, size_t byt
     prm.inner_max_iter = max_iter;
     prm.max_cycles = 1;
     prm.guard = x.f.guard;
+    prm.barrier_timeout_ns = grid_barrier_timeout_ns(grid);
     ADJ_TRY(launch_solve_begin(x));
     ADJ_TRY(launch_residual(x, prm));
+    // the solver form of the grid's own FP64 solves: on chip where it fits
+    bool on_chip = false;
+    if (x.auto_form) ADJ_TRY(launch_pcg_resident(x, prm, &on_chip));
+    if (on_chip) {
+      const bcm_status st = grid_read_err(grid);
+      if (st != BCM_OK) return st;
+    }
     int done = 0;
-    for (int it = 0; it < max_iter;) {
+    for (int it = 0; it < max_iter && !on_chip;) {
       ADJ_TRY(cudaMemcpyAsync(&done, x.g.flags, sizeof(int), cudaMemcpyDeviceToHost, s));
       ADJ_TRY(cudaStreamSynchronize(s));
       if (done) break;

@@ -67,7 +67,7 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 struct Layout {
   size_t u, v, w, us, vs, ws, nx, ny, nz, phi, ub, p, b, bid, near_, r, p0, p1, q, e, w1, s0, s1;
   size_t face, fcube;  // fused PCG face planes and per-cube records (mixed, 16^3 cubes)
-  size_t nb, aux, sim, lvl, ijk, w3, nbw3, slot, sp, ss, counter, flags, guard, bar, err;
+  size_t nb, aux, sim, lvl, ijk, w3, nbw3, slot, sp, ss, counter, flags, guard, bar, err, words;
   size_t total;
   size_t n_slots;
 };
@@ -472,6 +472,7 @@ Layout plan(const bcm_grid_desc* d, int n_slots, const MgHost& mg, MgLayout* ml)
   L.guard = take(64);
   L.bar = take(sizeof(unsigned int) * (kTicketWords + 32));
   L.err = take(64);
+  L.words = take(res_words_bytes(d->n_sims));
   if (mg.ok && ml) {  // multigrid preconditioner
     for (int l = 0; l <= mg.L; ++l) {
       ml->x[l] = take(mg.n[l] * V);
@@ -521,7 +522,7 @@ struct StepGraph {
   unsigned int counted[2] = {0, 0};  // body executions already in the launch count
   double rtol = 0.0;
   int max_iter = 0, cycles = 0;
-  int slabs_p = 0, single_pass = 0, resident = 0, fused = 0;  // the PCG launch shape captured
+  int slabs_p = 0, single_pass = 0, resident = 0, fused = 0, auto_form = 0;  // the PCG launch shape captured
   int slabs_m = -1;  // the momentum / right-hand-side slabs captured
   double inner_rtol = 0.0;
   int persistent_slabs = 0;
@@ -623,6 +624,9 @@ const Ctx* grid_ctx(const bcm_grid* g) { return &g->ctx; }
 int grid_two_level(const bcm_grid* g) { return g->T.two_level; }
 int grid_device(const bcm_grid* g) { return g->device; }
 cudaStream_t grid_stream(const bcm_grid* g) { return g->stream; }
+unsigned long long grid_barrier_timeout_ns(const bcm_grid* g) {
+  return (unsigned long long)(g->barrier_timeout_s * 1e9);
+}
 bcm_status grid_fail(bcm_status st, const char* msg) { return fail(st, "%s", msg); }
 }  // namespace bcm
 
@@ -731,6 +735,7 @@ extern "C" bcm_status bcm_create_grid(const bcm_grid_desc* desc, void* dev_works
   x.persistent = (!g->solve64 && desc->n_sims <= 256) ? 1 : 0;
   x.single_pass = 0;
   x.resident = 0;
+  x.auto_form = desc->n_sims <= 256 ? 1 : 0;
   x.fused = 0;  // the fused single-barrier form: selected by bcm_set_launch(5, ...)
   x.slabs_m = 0;  // the momentum / right-hand-side slab depth: bcm_set_stencil_slabs
   x.lag_bf16 = desc->lagged_bf16;
@@ -769,6 +774,7 @@ extern "C" bcm_status bcm_create_grid(const bcm_grid_desc* desc, void* dev_works
   F.guard = (unsigned int*)(W + L.guard);
   F.bar = (unsigned int*)(W + L.bar);
   F.err = (int*)(W + L.err);
+  F.words = W + L.words;
   x.use_mg = 0;
   x.mg = MgDev{};
   x.part = PartDev{};
@@ -962,6 +968,12 @@ bcm_status read_err(bcm_grid* g) {
   return BCM_OK;
 }
 
+}  // namespace
+namespace bcm {
+bcm_status grid_read_err(bcm_grid* g) { return read_err(g); }
+}  // namespace bcm
+namespace {
+
 // Inner FP32 reduction per defect-correction cycle.  Measured on the 4.2M-cell sphere
 // flow: restarting the inner CG every cycle works best at 1e-5 (3 cycles, ~1500
 // iterations per step); keeping its search direction (reliable updates) needs the FP64
@@ -1061,7 +1073,7 @@ bcm_status solve(bcm_grid* g, double rtol, int max_iter) {
     while (cycles < g->max_cycles) {
       for (int b = 0; b < batch && cycles < g->max_cycles; ++b, ++cycles) {
         RUN(BCM_K_PCG, launch_pcg(x, pin, &g->pcg_form));
-        if (g->pcg_form != PCG_STREAMING) RUN(BCM_K_ADD_CORRECTION, launch_add_correction(x));
+        if (!adds_correction(g->pcg_form)) RUN(BCM_K_ADD_CORRECTION, launch_add_correction(x));
         RUN(BCM_K_RESIDUAL, launch_residual(x, prm));
       }
       if ((st = read_flags(g, flags)) != BCM_OK) return st;
@@ -1070,6 +1082,15 @@ bcm_status solve(bcm_grid* g, double rtol, int max_iter) {
       batch = 1;
     }
     return BCM_OK;
+  }
+  if (g->solve64 && !mg && x.auto_form) {  // FP64 on chip where it fits, else two launches
+    bool launched = false;
+    RUN(BCM_K_PCG, launch_pcg_resident(x, prm, &launched));
+    if (launched) {
+      g->pcg_form = PCG_RESIDENT;
+      return read_err(g);
+    }
+    g->launch_count -= 1;
   }
   if ((st = read_flags(g, flags)) != BCM_OK) return st;
   if (g->solve64) {
@@ -1404,7 +1425,7 @@ bcm_status issue_graph_step(bcm_grid* g, cudaStream_t s, double rtol, int max_it
     pin.x64_add = x.f.p;
     for (int c = 0; c < cycles; ++c) {
       CUDA_TRY(launch_pcg(x, pin, &g->pcg_form));
-      if (g->pcg_form != PCG_STREAMING) CUDA_TRY(launch_add_correction(x));
+      if (!adds_correction(g->pcg_form)) CUDA_TRY(launch_add_correction(x));
       CUDA_TRY(launch_residual(x, prm));
     }
   }
@@ -1434,7 +1455,7 @@ extern "C" bcm_status bcm_step_graph(bcm_grid* g, int n_steps, double rtol, int 
   if (!sg.exec || sg.rtol != rtol || sg.max_iter != max_iter || sg.cycles != cycles ||
       sg.inner_rtol != g->inner_rtol || sg.recycle != g->recycle ||
       sg.slabs_p != g->ctx.slabs_p || sg.single_pass != g->ctx.single_pass ||
-      sg.resident != g->ctx.resident || sg.fused != g->ctx.fused || sg.gen != g->gen ||
+      sg.resident != g->ctx.resident || sg.auto_form != g->ctx.auto_form || sg.fused != g->ctx.fused || sg.gen != g->gen ||
       sg.mg != g->ctx.use_mg || (sg.mg && sg.cycles != g->max_cycles) ||
       sg.slabs_m != g->ctx.slabs_m) {
     bcm_status bst = graph_body_launches(g);  // the old loops' launches so far
@@ -1475,6 +1496,7 @@ extern "C" bcm_status bcm_step_graph(bcm_grid* g, int n_steps, double rtol, int 
     sg.slabs_p = g->ctx.slabs_p;
     sg.single_pass = g->ctx.single_pass;
     sg.resident = g->ctx.resident;
+    sg.auto_form = g->ctx.auto_form;
     sg.fused = g->ctx.fused;
     sg.gen = g->gen;
     sg.mg = g->ctx.use_mg;
@@ -1562,6 +1584,7 @@ extern "C" bcm_status bcm_set_launch(bcm_grid* g, int persistent, int slabs_a, i
   g->ctx.persistent = persistent ? 1 : 0;
   g->ctx.single_pass = persistent == 2 ? 1 : 0;
   g->ctx.resident = persistent == 3 ? 1 : 0;
+  g->ctx.auto_form = 0;
   g->ctx.fused = persistent == 5 ? 1 : 0;
   if (persistent) {
     g->ctx.slabs_p = slabs_a;

@@ -39,6 +39,7 @@ struct Fields {
   unsigned int* guard;    // graph-loop body counter
   unsigned int* bar;      // persistent PCG grid barrier words
   int* err;               // persistent PCG: a barrier wait timed out
+  void* words;            // on-chip PCG: the blocks' partial sums (res_words_bytes)
 };
 
 struct SolveParams {
@@ -59,7 +60,7 @@ struct SolveParams {
   // multigrid PCG inside a captured step: body executions of the inner and the outer
   // loop, counted on the device for the launch count ([0], [1]; cumulative)
   unsigned int* body_count;
-  // mixed mode, streaming persistent PCG: the FP64 iterate the kernel adds its FP32
+  // mixed mode, streaming and on-chip persistent PCG: the FP64 iterate the kernel adds its FP32
   // correction e to at the end of the inner solve (x64 += e, the defect correction's
   // update; the separate k_add_correction launch is then left out), or NULL
   double* x64_add;
@@ -118,7 +119,8 @@ struct Ctx {
   int slabs_p;  // persistent PCG: z-slabs per cube (1, 2 or 4)
   int persistent;  // 1: one cooperative launch per PCG solve; 0: two launches per iteration
   int single_pass; // persistent PCG: one pass and one grid barrier per iteration
-  int resident;    // persistent PCG: search direction in shared memory where it fits
+  int resident;    // persistent PCG: the on-chip form where it fits (FP32 inner solves)
+  int auto_form;   // no launch shape asked for: the on-chip form where it fits, in either type
   int fused;       // persistent PCG: the single-barrier form with bulk-copy staging
   int slabs_m;     // momentum and right-hand side: z-slabs per 16^3 cube (0: default)
   int lag_bf16;    // mixed mode: N^{n-1} stored as bfloat16
@@ -150,7 +152,12 @@ enum { PCG_TWO_LAUNCH = 0, PCG_STREAMING = 1, PCG_SINGLE_PASS = 2, PCG_RESIDENT 
 // The persistent PCG in the form the launch shape and the grid select; *form gets it.
 cudaError_t launch_pcg(const Ctx& x, const SolveParams& prm, int* form);
 cudaError_t launch_pcg1(const Ctx& x, const SolveParams& prm);
+// The on-chip form; *launched = false when the grid does not fit it.  In mixed mode it adds
+// its correction to the FP64 iterate (SolveParams::x64_add), like the streaming form.
 cudaError_t launch_pcg_resident(const Ctx& x, const SolveParams& prm, bool* launched);
+cudaError_t launch_pcg_resident64(const Ctx& x, const SolveParams& prm, bool* launched);
+size_t res_words_bytes(int n_sims);
+inline bool adds_correction(int form) { return form == PCG_STREAMING || form == PCG_RESIDENT; }
 // The fused single-barrier form (FP32 inner solve, 16^3 cubes); *launched = false when
 // the grid does not fit it (the caller falls back to the streaming form).
 cudaError_t launch_pcg_fused(const Ctx& x, const SolveParams& prm, bool* launched);

@@ -441,6 +441,15 @@ static cudaError_t pcg_dispatch(const Ctx& x, const SolveParams& prm, TX* xv) {
 
 cudaError_t launch_pcg(const Ctx& x, const SolveParams& prm, int* form) {
   if (x.g.n_sims > kMaxPersistentSims) return cudaErrorInvalidValue;
+  // the on-chip form wherever the vectors fit, unless a launch shape was asked for
+  if (x.auto_form || (x.resident && x.slabs_p == 1 && !x.solve64)) {
+    bool launched = false;
+    const cudaError_t e = launch_pcg_resident(x, prm, &launched);
+    if (e != cudaSuccess || launched) {
+      *form = PCG_RESIDENT;
+      return e;
+    }
+  }
   // every launch starts its grid barrier's arrival counter at zero
   {
     const cudaError_t e = cudaMemsetAsync(x.f.bar + 32, 0, 32 * sizeof(unsigned int), x.stream);
@@ -457,14 +466,6 @@ cudaError_t launch_pcg(const Ctx& x, const SolveParams& prm, int* form) {
   if (x.single_pass) {
     *form = PCG_SINGLE_PASS;
     return launch_pcg1(x, prm);
-  }
-  if (x.resident && x.slabs_p == 1) {
-    bool launched = false;
-    const cudaError_t e = launch_pcg_resident(x, prm, &launched);
-    if (e != cudaSuccess || launched) {
-      *form = PCG_RESIDENT;
-      return e;
-    }
   }
   *form = PCG_STREAMING;
   return x.solve64 ? pcg_dispatch<double, double>(x, prm, x.f.p)
