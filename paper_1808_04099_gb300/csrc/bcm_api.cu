@@ -86,7 +86,7 @@ int face_axis(int f) { return f >> 1; }
 struct MgAgg {
   int n = 0;                          // nodes
   std::vector<int> row, col, cptr, cidx, parent;
-  std::vector<double> val, diag;
+  std::vector<double> val, diag, inv;
 };
 struct MgHost {
   bool ok = false;
@@ -96,7 +96,7 @@ struct MgHost {
 };
 struct MgLayout {
   size_t x[kMgMaxL + 1], y[kMgMaxL + 1], r[kMgMaxL + 1], rr;
-  size_t ar[kMgMaxM], ax[kMgMaxM], at[kMgMaxM], diag[kMgMaxM], val[kMgMaxM];
+  size_t ar[kMgMaxM], ax[kMgMaxM], at[kMgMaxM], as[kMgMaxM], diag[kMgMaxM], val[kMgMaxM], inv[kMgMaxM];
   size_t row[kMgMaxM], col[kMgMaxM], cptr[kMgMaxM], cidx[kMgMaxM], parent[kMgMaxM];
 };
 
@@ -387,6 +387,7 @@ MgHost mg_build(const bcm_grid_desc* d, const HostTables& T) {
         dsum += e.second;
       }
       g.diag.push_back(dsum);
+      g.inv.push_back(dsum > 0.0 ? kMgOmega * (1.0 / dsum) : 0.0);
       g.row.push_back((int)g.col.size());
       for (int u : kids[U]) g.cidx.push_back(u);
       g.cptr.push_back((int)g.cidx.size());
@@ -475,7 +476,8 @@ Layout plan(const bcm_grid_desc* d, int n_slots, const MgHost& mg, MgLayout* ml)
   L.words = take(res_words_bytes(d->n_sims));
   if (mg.ok && ml) {  // multigrid preconditioner
     for (int l = 0; l <= mg.L; ++l) {
-      ml->x[l] = take(mg.n[l] * V);
+      // levels on quad tiles form x = S r where they need it
+      ml->x[l] = take(d->cells_per_edge >> l >= 8 ? 0 : mg.n[l] * V);
       ml->y[l] = take(mg.n[l] * V);
       ml->r[l] = l ? take(mg.n[l] * V) : 0;
     }
@@ -486,7 +488,9 @@ Layout plan(const bcm_grid_desc* d, int n_slots, const MgHost& mg, MgLayout* ml)
       ml->ar[k] = take(a.n * 8);
       ml->ax[k] = take(a.n * 8);
       ml->at[k] = take(a.n * 8);
+      ml->as[k] = take(a.n * 8);
       ml->diag[k] = take(a.n * 8);
+      ml->inv[k] = take(a.n * 8);
       ml->val[k] = take(a.val.size() * 8);
       ml->row[k] = take((a.n + 1) * sizeof(int));
       ml->col[k] = take(a.col.size() * sizeof(int));
@@ -711,6 +715,7 @@ extern "C" bcm_status bcm_create_grid(const bcm_grid_desc* desc, void* dev_works
   for (size_t k = 0; mgh.ok && k < mgh.agg.size(); ++k) {
     const MgAgg& a = mgh.agg[k];
     UP(ml.diag[k], a.diag.data(), a.diag.size() * sizeof(double));
+    UP(ml.inv[k], a.inv.data(), a.inv.size() * sizeof(double));
     if (!a.val.empty()) UP(ml.val[k], a.val.data(), a.val.size() * sizeof(double));
     UP(ml.row[k], a.row.data(), a.row.size() * sizeof(int));
     if (!a.col.empty()) UP(ml.col[k], a.col.data(), a.col.size() * sizeof(int));
@@ -797,7 +802,9 @@ extern "C" bcm_status bcm_create_grid(const bcm_grid_desc* desc, void* dev_works
       D.ar[k] = (double*)(W + ml.ar[k]);
       D.ax[k] = (double*)(W + ml.ax[k]);
       D.at[k] = (double*)(W + ml.at[k]);
+      D.as[k] = (double*)(W + ml.as[k]);
       D.diag[k] = (double*)(W + ml.diag[k]);
+      D.inv[k] = (double*)(W + ml.inv[k]);
       D.val[k] = (double*)(W + ml.val[k]);
       D.row[k] = (int*)(W + ml.row[k]);
       D.col[k] = (int*)(W + ml.col[k]);

@@ -399,6 +399,11 @@ __device__ __forceinline__ double ld_acc(const double* p) { return __ldcg(p); }
 __device__ __forceinline__ void acc_add(SimState& st, int idx, double v) {
   atomicAdd(&st.acc[blockIdx.x % kStripes][idx], v);
 }
+// The same for kernels whose blocks hold several cubes: the stripe of cube c, as if each cube
+// had a block of its own (few cubes per stripe keep the sums' order, hence their bits).
+__device__ __forceinline__ void acc_add_cube(SimState& st, int idx, int c, double v) {
+  atomicAdd(&st.acc[c % kStripes][idx], v);
+}
 // Sum of accumulator idx over the stripes, which are reset to zero (last block only).
 __device__ __forceinline__ double acc_take(SimState& st, int idx) {
   double s = 0.0;

@@ -83,8 +83,9 @@ struct MgDev {
   void* rr;              // level L: residual after pre-smoothing, one value per cube
   int n[kMgMaxM];        // nodes of aggregate level k
   int nnz[kMgMaxM];      // off-diagonal entries of level k
-  double *ar[kMgMaxM], *ax[kMgMaxM], *at[kMgMaxM];  // residual, iterate, scratch
+  double *ar[kMgMaxM], *ax[kMgMaxM], *at[kMgMaxM], *as[kMgMaxM];  // residual, result, scratch
   double *diag[kMgMaxM], *val[kMgMaxM];              // K: diagonal, -off-diagonal (CSR)
+  double* inv[kMgMaxM];                // omega / diagonal (0 where the diagonal is 0)
   int *row[kMgMaxM], *col[kMgMaxM];
   int *cptr[kMgMaxM], *cidx[kMgMaxM];  // children: level k-1 nodes (cubes for k = 0)
   int *parent[kMgMaxM];                // parent at level k of each level k-1 node

@@ -20,12 +20,19 @@
 //   V_l(r) = x + S (r - K x),  x = S r + s P V_{l+1}(P^T (r - K S r)),
 //   V_top(r) = four damped-Jacobi sweeps from zero.
 //
-// Launches per V-cycle: one per per-cube level on the way down (pre-smoothing with the
-// neighbours' values computed on the fly, residual, restriction), one single-block
-// launch for the aggregate levels, and one per per-cube level on the way up
-// (prolongation of the neighbours on the fly, post-smoothing).  The last launch also
-// forms <r, z> per sim and, after PCG pass B, takes the iteration's decisions (beta,
-// convergence) that pass B leaves to it.
+// Launches per V-cycle: the levels of 16^3 and 8^3 cells per cube on quad tiles
+// (bcm_quad.cuh), the 4^3 and 2^3 levels of larger grids with a thread per cell, the rest
+// down to one node per sim and back up in one launch of a cluster, and after the finest up
+// launch the PCG's decisions (beta, convergence).  After pass A the finest down launch also
+// does the PCG's pass B.
+//
+// What bounds it: the finest level moves 49 bytes a cell and iteration in FP32 (pass A 16,
+// down with pass B 24.5, up 8.5; 60 before, when x = S r was stored and read).  On 83M cells
+// (two levels) the three launches take 281, 405 and 277 us, 4.7, 5.0 and 2.5 TB/s (427, 470
+// and 410 us with padded tiles); on 4.2M cells 19.5, 25 and 19 us (31, 31, 39).  In FP64
+// they are bound by the FP64 pipe: 96, 131 and 122 us (138, 192, 151).  Below the finest
+// level it is latency: 5 launches, 58 us serialised at 1024 cubes, where there were 9 in 80.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -34,6 +41,7 @@
 #include "bcm_internal.cuh"
 #include "bcm_kernels.h"
 #include "bcm_persist.cuh"
+#include "bcm_quad.cuh"
 
 namespace bcm {
 
@@ -118,6 +126,46 @@ __device__ __forceinline__ TV mg_across(const DevGrid& g, int c, int l, int i, i
   return TV(0.25) * sum;
 }
 
+// The sum over the six faces of w (xc - value across) for cell (i, j, k) of cube c, with every
+// load of the cell in flight before the first use: the six face entries, then the six
+// values at(cube, cell).  (Face by face, each behind its own branch, they are twelve
+// dependent round trips: 4-9k cycles a level however few the cells.)  2:1 faces go through
+// mg_across.
+template <int BL, class TV, class At>
+__device__ __forceinline__ TV mg_faces(const DevGrid& g, int c, int l, int i, int j, int k, TV xc,
+                                       const At& at) {
+  int nb[6];
+#pragma unroll
+  for (int f = 0; f < 6; ++f) nb[f] = checked_nb(g, g.nb[6 * c + f]);
+  TV v[6];
+  unsigned edge = 0u;
+#pragma unroll
+  for (int f = 0; f < 6; ++f) {
+    int q[3] = {i, j, k};
+    const int d = f >> 1, side = f & 1, o = q[d];
+    const bool out = side ? o == BL - 1 : o == 0;
+    if (out) edge |= 1u << f;
+    const bool other = out && nb[f] >= 0;
+    q[d] = out ? (other ? (side ? 0 : BL - 1) : o) : (side ? o + 1 : o - 1);
+    v[f] = at(other ? nb[f] : c, lcell<BL>(q[0], q[1], q[2]));
+  }
+  TV acc = TV(0);
+#pragma unroll
+  for (int f = 0; f < 6; ++f) {
+    TV w = TV(1);
+    if ((edge >> f & 1u) && nb[f] < 0) {
+      if (nb[f] == NB_BOUNDARY) {
+        v[f] = g.sp[g.sim[c]].bc[f] == BC_OUTFLOW ? -xc : xc;
+      } else {
+        auto val = [&](int cube, int a, int b, int e) { return at(cube, lcell<BL>(a, b, e)); };
+        v[f] = mg_across<BL, TV>(g, c, l, i, j, k, f, xc, val, w);
+      }
+    }
+    acc += w * (xc - v[f]);
+  }
+  return acc;
+}
+
 // omega / diag(K_l) of cell (i, j, k) of cube c on per-cube level l (BL cells per edge):
 // diag(K_l) = 4^l diag(K) of a fine cell with the same boundary faces; wscale =
 // omega / 4^l.  Neighbouring cubes belong to the same sim, so sp serves them too.
@@ -127,70 +175,27 @@ __device__ __forceinline__ TV smooth_w(const DevGrid& g, const SimParams& sp, in
   return wscale * sim_inv<TV>(sp, g.lvl[c], s3_of<BL>(g.w3 + 6 * c, i, j, k));
 }
 
-// ---- down: x = S r, rr = r - K x, restriction of rr (P^T: sums)
-// One thread per coarse cell (its 2x2x2 fine cells), or per cube on the level with one
-// cell per cube (its residual goes to `rc` per cube for the aggregate levels).
+// ---- down: x = S r, rr = r - K x, restriction of rr (P^T: sums), on levels of 4^3 and 2^3
+// cells per cube that are too large for the coarse kernel below.
+// One thread per fine cell: the eight children of a coarse cell are eight consecutive
+// threads of one warp (child bits in the low three bits of the thread index), so the
+// restriction is a three-step shuffle sum.  Threads of finished sims and of the tail take
+// part in the shuffles with zeros.
+// GIVEN: x = S r was formed by the finer level's launch, which knows each coarse cell once,
+// where its six neighbours would each form it again (a launch of this kernel spends most
+// of its instructions on that); else (the finest level of 4^3 cubes) it is formed here and
+// stored.  The launch forms the next level's x the same way.
 template <int BL, class TV>
-__device__ __forceinline__ void mg_down_item(const DevGrid& g, int l, TV wscale, TV cscale,
-                                             const TV* __restrict__ r, TV* __restrict__ x,
-                                             TV* __restrict__ rc, int all, long long t) {
-  constexpr int CB = BL > 1 ? BL / 2 : 1, C3 = CB * CB * CB, B3 = BL * BL * BL;
-  constexpr int CH = BL > 1 ? 2 : 1;
-  const int c = (int)(t / C3), ci = (int)(t - (long long)c * C3);
-  const int s = g.sim[c];
-  if (!all && g.ss[s].done) return;
-  const int I = ci % CB, J = (ci / CB) % CB, Kc = ci / (CB * CB);
-  const SimParams& sp = g.sp[s];
-  const TV coef = cube_h<TV>(g, sp, c) * cscale;  // 4^l h
-  auto sval = [&](int cube, int ci2, int cj2, int ck2) {
-    return smooth_w<BL, TV>(g, sp, cube, ci2, cj2, ck2, wscale) *
-           r[(size_t)cube * B3 + lcell<BL>(ci2, cj2, ck2)];
-  };
-  TV sum = TV(0);
-#pragma unroll
-  for (int dk = 0; dk < CH; ++dk)
-#pragma unroll
-    for (int dj = 0; dj < CH; ++dj)
-#pragma unroll
-      for (int di = 0; di < CH; ++di) {
-        const int i = CH * I + di, j = CH * J + dj, k = CH * Kc + dk;
-        const size_t gi = (size_t)c * B3 + lcell<BL>(i, j, k);
-        const TV rv = r[gi];
-        const TV xc = smooth_w<BL, TV>(g, sp, c, i, j, k, wscale) * rv;
-        TV acc = TV(0);
-#pragma unroll
-        for (int f = 0; f < 6; ++f) {
-          TV w;
-          const TV xn = mg_across<BL, TV>(g, c, l, i, j, k, f, xc, sval, w);
-          acc += w * (xc - xn);
-        }
-        x[gi] = xc;
-        sum += rv - coef * acc;
-      }
-  rc[t] = sum;
+__device__ __forceinline__ TV next_x(const DevGrid& g, const SimParams& sp, int c, int I, int J,
+                                     int K, TV wscale, TV rc) {
+  constexpr int CB = BL / 2;
+  return smooth_w<CB, TV>(g, sp, c, I, J, K, TV(0.25) * wscale) * rc;
 }
-
-template <int BL, class TV>
-__global__ __launch_bounds__(256) void k_mg_down(DevGrid g, int l, TV wscale, TV cscale,
-                                                 const TV* __restrict__ r,
-                                                 TV* __restrict__ x, TV* __restrict__ rc,
-                                                 int all) {
-  cudaGridDependencySynchronize();  // launched after the previous level's kernel
-  constexpr int CB = BL > 1 ? BL / 2 : 1;
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)g.n_cubes * CB * CB * CB) return;
-  mg_down_item<BL, TV>(g, l, wscale, cscale, r, x, rc, all, t);
-}
-
-// The same with one thread per fine cell (BL >= 2): the eight children of a coarse cell
-// are eight consecutive threads of one warp (child bits in the low three bits of the
-// thread index), so the restriction is a three-step shuffle sum.  Threads of finished
-// sims and of the tail take part in the shuffles with zeros.
-template <int BL, class TV>
+template <int BL, class TV, bool GIVEN>
 __global__ __launch_bounds__(256) void k_mg_down_cell(DevGrid g, int l, TV wscale, TV cscale,
                                                       const TV* __restrict__ r,
                                                       TV* __restrict__ x, TV* __restrict__ rc,
-                                                      int all) {
+                                                      TV* __restrict__ xn, int all) {
   cudaGridDependencySynchronize();  // launched after the previous level's kernel
   static_assert(BL >= 2, "restriction over 2x2x2 children");
   constexpr int CB = BL / 2, C3 = CB * CB * CB, B3 = BL * BL * BL;
@@ -198,75 +203,54 @@ __global__ __launch_bounds__(256) void k_mg_down_cell(DevGrid g, int l, TV wscal
   const long long total = (long long)g.n_cubes * B3;
   const int c = (int)(t / B3), q = (int)(t - (long long)c * B3);
   const int d = q & 7, ci = q >> 3;
+  const int I = ci % CB, J = (ci / CB) % CB, Kc = ci / (CB * CB);
+  const bool on = t < total && (all || !g.ss[g.sim[c]].done);
   TV val = TV(0);
-  if (t < total && (all || !g.ss[g.sim[c]].done)) {
-    const int I = ci % CB, J = (ci / CB) % CB, Kc = ci / (CB * CB);
+  if (on) {
     const int i = 2 * I + (d & 1), j = 2 * J + ((d >> 1) & 1), k = 2 * Kc + (d >> 2);
     const SimParams& sp = g.sp[g.sim[c]];
     const TV coef = cube_h<TV>(g, sp, c) * cscale;
     const size_t gi = (size_t)c * B3 + lcell<BL>(i, j, k);
     const TV rv = r[gi];
-    const TV xc = smooth_w<BL, TV>(g, sp, c, i, j, k, wscale) * rv;
-    auto sval = [&](int cube, int ci2, int cj2, int ck2) {
-      return smooth_w<BL, TV>(g, sp, cube, ci2, cj2, ck2, wscale) *
-             r[(size_t)cube * B3 + lcell<BL>(ci2, cj2, ck2)];
+    auto sval = [&](int cube, int cell) {
+      const size_t gn = (size_t)cube * B3 + cell;
+      if constexpr (GIVEN) return x[gn];
+      else
+        return smooth_w<BL, TV>(g, sp, cube, cell % BL, (cell / BL) % BL, cell / (BL * BL), wscale) *
+               r[gn];
     };
-    TV acc = TV(0);
-#pragma unroll
-    for (int f = 0; f < 6; ++f) {
-      TV w;
-      const TV xn = mg_across<BL, TV>(g, c, l, i, j, k, f, xc, sval, w);
-      acc += w * (xc - xn);
-    }
-    x[gi] = xc;
+    const TV xc = sval(c, lcell<BL>(i, j, k));
+    const TV acc = mg_faces<BL, TV>(g, c, l, i, j, k, xc, sval);
+    if constexpr (!GIVEN) x[gi] = xc;
     val = rv - coef * acc;
   }
   val += __shfl_xor_sync(0xffffffffu, val, 1);
   val += __shfl_xor_sync(0xffffffffu, val, 2);
   val += __shfl_xor_sync(0xffffffffu, val, 4);
-  if (d == 0 && t < total && (all || !g.ss[g.sim[c]].done)) rc[(size_t)c * C3 + ci] = val;
+  if (d == 0 && on) {
+    rc[(size_t)c * C3 + ci] = val;
+    xn[(size_t)c * C3 + ci] = next_x<BL, TV>(g, g.sp[g.sim[c]], c, I, J, Kc, wscale, val);
+  }
 }
 
 // ---- up: x~ = x + P y_coarse (on the fly for the cell and its neighbours), then
-// y = x~ + S (r - K x~).  One thread per cell.  On the level with one cell per cube the
-// coarse values come from aggregate level 0 (FP64, through the cube's parent).
-template <int BL, class TV>
-__device__ __forceinline__ TV up_value(const TV* __restrict__ x, const TV* __restrict__ yc,
-                                       const double* __restrict__ yagg,
-                                       const int* __restrict__ agg_parent, int c, int i, int j,
-                                       int k) {
-  constexpr int B3 = BL * BL * BL;
-  const TV xv = x[(size_t)c * B3 + lcell<BL>(i, j, k)];
-  if constexpr (BL == 1) {
-    return xv + TV(kMgOver * yagg[agg_parent[c]]);
-  } else {
-    constexpr int CB = BL / 2;
-    return xv + TV(kMgOver) * yc[(size_t)c * CB * CB * CB + lcell<CB>(i >> 1, j >> 1, k >> 1)];
-  }
-}
-
+// y = x~ + S (r - K x~).  One thread per cell.
 template <int BL, class TV>
 __device__ __forceinline__ TV up_cell(const DevGrid& g, int l, TV wscale, TV cscale,
-                                      const TV* __restrict__ r,
-                                      const TV* __restrict__ x, const TV* __restrict__ yc,
-                                      const double* __restrict__ yagg,
-                                      const int* __restrict__ agg_parent, int c, int i, int j,
-                                      int k, TV* rv_out) {
-  constexpr int B3 = BL * BL * BL;
+                                      const TV* __restrict__ r, const TV* __restrict__ x,
+                                      const TV* __restrict__ yc, int c, int i, int j, int k,
+                                      TV* rv_out) {
+  constexpr int B3 = BL * BL * BL, CB = BL / 2;
   const SimParams& sp = g.sp[g.sim[c]];
   const TV coef = cube_h<TV>(g, sp, c) * cscale;
-  const TV xc = up_value<BL, TV>(x, yc, yagg, agg_parent, c, i, j, k);
-  auto uval = [&](int cube, int ci2, int cj2, int ck2) {
-    return up_value<BL, TV>(x, yc, yagg, agg_parent, cube, ci2, cj2, ck2);
+  auto uval = [&](int cube, int cell) {
+    const int a = cell % BL, b = (cell / BL) % BL, e = cell / (BL * BL);
+    return x[(size_t)cube * B3 + cell] +
+           TV(kMgOver) * yc[(size_t)cube * CB * CB * CB + lcell<CB>(a >> 1, b >> 1, e >> 1)];
   };
-  TV acc = TV(0);
-#pragma unroll
-  for (int f = 0; f < 6; ++f) {
-    TV w;
-    const TV xn = mg_across<BL, TV>(g, c, l, i, j, k, f, xc, uval, w);
-    acc += w * (xc - xn);
-  }
   const TV rv = r[(size_t)c * B3 + lcell<BL>(i, j, k)];
+  const TV xc = uval(c, lcell<BL>(i, j, k));
+  const TV acc = mg_faces<BL, TV>(g, c, l, i, j, k, xc, uval);
   *rv_out = rv;
   return xc + smooth_w<BL, TV>(g, sp, c, i, j, k, wscale) * (rv - coef * acc);
 }
@@ -275,15 +259,13 @@ template <int BL, class TV>
 __device__ __forceinline__ void mg_up_item(const DevGrid& g, int l, TV wscale, TV cscale,
                                            const TV* __restrict__ r, const TV* __restrict__ x,
                                            const TV* __restrict__ yc,
-                                           const double* __restrict__ yagg,
-                                           const int* __restrict__ agg_parent,
                                            TV* __restrict__ y, int all, long long t) {
   constexpr int B3 = BL * BL * BL;
   const int c = (int)(t / B3), cell = (int)(t - (long long)c * B3);
   if (!all && g.ss[g.sim[c]].done) return;
   const int i = cell % BL, j = (cell / BL) % BL, k = cell / (BL * BL);
   TV rv;
-  y[t] = up_cell<BL, TV>(g, l, wscale, cscale, r, x, yc, yagg, agg_parent, c, i, j, k, &rv);
+  y[t] = up_cell<BL, TV>(g, l, wscale, cscale, r, x, yc, c, i, j, k, &rv);
 }
 
 template <int BL, class TV>
@@ -291,13 +273,11 @@ __global__ __launch_bounds__(256) void k_mg_up(DevGrid g, int l, TV wscale, TV c
                                                const TV* __restrict__ r,
                                                const TV* __restrict__ x,
                                                const TV* __restrict__ yc,
-                                               const double* __restrict__ yagg,
-                                               const int* __restrict__ agg_parent,
                                                TV* __restrict__ y, int all) {
   cudaGridDependencySynchronize();  // launched after the previous level's kernel
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long long)g.n_cubes * BL * BL * BL) return;
-  mg_up_item<BL, TV>(g, l, wscale, cscale, r, x, yc, yagg, agg_parent, y, all, t);
+  mg_up_item<BL, TV>(g, l, wscale, cscale, r, x, yc, y, all, t);
 }
 
 // The last block of the finest up launch: mode 0 (start of a solve) takes <r, z> as
@@ -313,9 +293,9 @@ __device__ void mg_decide(const DevGrid& g, const SolveParams& prm, int mode, in
       alive |= !t.done;
       continue;
     }
-    const double rr = acc_take(t, ACC_RR);
+    const double rr = acc_take(t, ACC_RR), pq = acc_take(t, ACC_PQ);
     if (t.done) continue;
-    if (t.nonfinite || !isfinite(rr) || !isfinite(rzs)) {
+    if (t.nonfinite || !isfinite(rr) || !isfinite(rzs) || !isfinite(pq)) {
       t.nonfinite = 1;
       t.done = 1;
       continue;
@@ -356,8 +336,6 @@ template <int B, int NT, class TV>
 __global__ __launch_bounds__(NT) void k_mg_up0(DevGrid g, const TV* __restrict__ r,
                                               const TV* __restrict__ x,
                                               const TV* __restrict__ yc,
-                                              const double* __restrict__ yagg,
-                                              const int* __restrict__ agg_parent,
                                               TV* __restrict__ z, SolveParams prm, int mode) {
   cudaGridDependencySynchronize();  // launched after the previous level's kernel
   constexpr int B3 = B * B * B, PER = B3 / NT;
@@ -372,7 +350,7 @@ __global__ __launch_bounds__(NT) void k_mg_up0(DevGrid g, const TV* __restrict__
     const int cell = (blockIdx.x - c * PER) * NT + threadIdx.x;
     const int i = cell % B, j = (cell / B) % B, k = cell / (B * B);
     TV rv;
-    const TV zv = up_cell<B, TV>(g, 0, TV(kMgOmega), TV(1), r, x, yc, yagg, agg_parent, c, i, j,
+    const TV zv = up_cell<B, TV>(g, 0, TV(kMgOmega), TV(1), r, x, yc, c, i, j,
                                  k, &rv);
     z[(size_t)c * B3 + cell] = zv;
     rz = double(rv * zv);
@@ -384,13 +362,12 @@ __global__ __launch_bounds__(NT) void k_mg_up0(DevGrid g, const TV* __restrict__
   if (last_block(g.counter)) mg_decide(g, prm, mode, NT);
 }
 
-// ---- levels of 8^3 / 16^3 cells per cube, one block per cube with the (B+2)^3 tile of
-// the PCG passes: down stages x = S r with the face halo, marches each column for
-// rr = r - K x and sums the 2x2x2 children of rr into r_{l+1}; up stages
-// x~ = x + s P y_{l+1}, marches for y = x~ + S (r - K x~) and, on the finest level, forms
-// <r, z>.  On level l, S = (omega / 4^l) D^-1 and K = 4^l h (sum of differences) with
-// the finest level's D: the launch passes wl = omega / 4^l and cl = 4^l.  Same values as
-// the per-cell kernels above.
+// ---- levels of 8^3 / 16^3 cells per cube on quad tiles (bcm_quad.cuh): down stages
+// x = S r with the face halo, forms rr = r - K x and sums its 2x2x2 children into r_{l+1};
+// up stages x~ = S r + s P y_{l+1} (S r formed again from r: cheaper than storing and
+// reading x), then y = x~ + S (r - K x~) and, on the finest level, <r, z>.  On level l,
+// S = (omega / 4^l) D^-1 and K = 4^l h (sum of differences) with the finest level's D: the
+// launch passes wl = omega / 4^l and cl = 4^l.  Same values as the per-cell kernels above.
 //
 // With FB the down launch also does the PCG's pass B (x_pcg += alpha p, r -= alpha q,
 // <r, r>): it reads the residual r_in of the iteration and writes the new one to the
@@ -404,23 +381,41 @@ struct PassB {
   TV *ra, *rb;           // residual: in ra, out rb at even iterations; swapped at odd
 };
 
+// alpha = <r, z> / <p, K p> of one sim (zero where the denominator is zero or not finite)
+template <class TV>
+__device__ __forceinline__ double cg_alpha_of(double rz, double pq) {
+  return pq != 0.0 && isfinite(pq) ? quick_div<TV>(rz, pq, quick_rcp<TV>(pq)) : 0.0;
+}
+
 template <int B, class TV, bool FB>
-__global__ __launch_bounds__(B * B) void k_mg_down0_tile(DevGrid g, const TV* __restrict__ r0,
-                                                         TV* __restrict__ x,
-                                                         TV* __restrict__ r1, int all,
-                                                         PassB<TV> pb, TV wl, TV cl, int lsh) {
-  cudaGridDependencySynchronize();  // launched after the previous level's kernel
-  using SL = Slab<B, B>;
-  constexpr int NT = B * B, B3 = B * B * B, BB = B * B, PP = SL::P * SL::P, CB = B / 2;
+__global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_down_quad(DevGrid g, const TV* __restrict__ r0,
+                                                            TV* __restrict__ r1,
+                                                            TV* __restrict__ x1, int all,
+                                                            PassB<TV> pb, TV wl, TV cl, int lsh) {
+  using T = QT<B>;
+  constexpr int B3 = T::B3, BB = T::BB, CB = B / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  TV* S = reinterpret_cast<TV*>(smem_raw);
-  TV* RR = S + (SL::N + 3) / 4 * 4;
-  __shared__ CubeSh<TV> cs;
-  __shared__ double red[32];
-  const int c = blockIdx.x;
-  SimState& st = g.ss[g.sim[c]];
+  __shared__ CubeQ<TV> cqs[T::CPB];
+  __shared__ TV alphas[T::CPB];
+  const int cub = threadIdx.x / T::TPC, lt = threadIdx.x - cub * T::TPC;
+  const int c = blockIdx.x * T::CPB + cub;
+  TV* S = reinterpret_cast<TV*>(smem_raw) + cub * T::N;
+  TV* gh = S + B3;
+  CubeQ<TV>& cq = cqs[cub];
+  const bool valid = c < g.n_cubes;
+  const CubeLoad L = cube_lookup(g, valid ? c : 0, lt);
+  Halo<B> H;
+  H.lookup(g, valid ? c : 0, lt);
+  cudaGridDependencySynchronize();  // launched after the previous level's kernel
+  poison_tile(reinterpret_cast<TV*>(smem_raw), T::CPB * T::N);
+  if (!valid) return;
+  SimState& st = g.ss[L.s];
+  double pq = 0.0, rz = 0.0;
+  if constexpr (FB) {  // the stripes of <p, K p>, and <r, z>
+    if (lt < kStripes) pq = ld_acc(&st.acc[lt][ACC_PQ]);
+    rz = st.rz;
+  }
   if (!all && st.done) return;
-  load_cube(cs, g, c);
   const TV* __restrict__ r = r0;
   TV* __restrict__ rout = nullptr;
   const TV* __restrict__ pn = nullptr;
@@ -430,375 +425,569 @@ __global__ __launch_bounds__(B * B) void k_mg_down0_tile(DevGrid g, const TV* __
     r = (it & 1) ? pb.rb : pb.ra;
     rout = (it & 1) ? pb.ra : pb.rb;
     pn = (it & 1) ? pb.p0 : pb.p1;
-    alpha = st.nonfinite ? TV(0) : TV(st.alpha);
   }
-  __syncthreads();
-  const TV w = wl;
-  TV rr2 = TV(0);
-  // the iteration's residual of a cell: r (FB: r_in - alpha q)
-  auto res = [&](size_t gi) {
-    if constexpr (FB) return r[gi] - alpha * pb.q[gi];
-    else return r[gi];
+  const int pos = lt % T::Q, i0 = (4 * pos) % B, j = (4 * pos) / B, k0 = 4 * (lt / T::Q);
+  const int cell0 = (k0 * B + j) * B + i0;
+  const size_t base = (size_t)c * B3 + cell0;
+  TV res[4][4], v[4][4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    ld4(r + base + m * BB, res[m]);
+    if constexpr (FB) ld4(pb.q + base + m * BB, v[m]);
+  }
+  TV ha[Halo<B>::R][4], hb[FB ? Halo<B>::R : 1][4];
+  H.each(lt, [&](int u, int, int n, int cell, int stride) {
+    const size_t gi = (size_t)n * B3 + cell;
+    ldq(r + gi, stride, ha[u]);
+    if constexpr (FB) ldq(pb.q + gi, stride, hb[u]);
+  });
+  cube_publish(cq, g, L, lt);
+  if constexpr (FB) {  // alpha, by the cube's first warp while the cells are in flight
+    if (lt < 32) {
+#pragma unroll
+      for (int o = 1; o < kStripes; o <<= 1) pq += __shfl_xor_sync(0xffffffffu, pq, o);
+      if (lt == 0) alphas[cub] = TV(cg_alpha_of<TV>(rz, pq));
+    }
+  }
+  T::sync();
+  if constexpr (FB) alpha = alphas[cub];
+  // S times the iteration's residual (FB: r_in - alpha q) on the halo
+  auto make = [&](int u, int f, int, int cell, int stride, TV (&o)[4]) {
+    TV inv[4];
+    if constexpr (FB) axpy4(-alpha, hb[u], ha[u], ha[u]);
+    nb_inv<B>(cq, g, c, f, cell, stride, inv);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) o[e] = (wl * inv[e]) * ha[u][e];
   };
-  auto val4 = [&](int cube, int cell0, int face, TV (&v)[4]) {
-    const size_t gi = (size_t)cube * B3 + cell0;
-    TV rr[4];
-    ld4(r + gi, rr);
+  auto one = [&](int n, int cell) {
+    const size_t gi = (size_t)n * B3 + cell;
+    TV x = r[gi];
+    if constexpr (FB) x -= alpha * pb.q[gi];
+    return wl * inv_diag_any<B, TV>(g, n, cell) * x;
+  };
+  H.store(gh, g, c, lt, make, one, lsh);
+  TV rr2 = TV(0);
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
     if constexpr (FB) {
-      TV qv[4];
-      ld4(pb.q + gi, qv);
+      axpy4(-alpha, v[m], res[m], res[m]);
+      rr2 += dot4(res[m], res[m]);
+      st4(rout + base + m * BB, res[m]);
+    }
+    TV inv[4];
+    quad_inv<B>(cq, i0, j, k0 + m, inv);
 #pragma unroll
-      for (int m = 0; m < 4; ++m) rr[m] = rr[m] - alpha * qv[m];
-      if (face < 0) {  // own cells: pass B
-        TV xv[4], pv[4];
-        ld4(pb.x + gi, xv);
-        ld4(pn + gi, pv);
+    for (int e = 0; e < 4; ++e) v[m][e] = (wl * inv[e]) * res[m][e];
+    own_quad<B>(S, gh, cq, i0, j, k0 + m, v[m]);
+  }
+  T::sync();
+  const TV h = cq.h * cl;
+  quad_column<B>(S, gh, cq, i0, j, k0, v,
+                 [&](int m, const TV (&acc)[4]) { axpy4(-h, acc, res[m], res[m]); });
+  // 2x2x2 sums: planes and x within the thread, y from the lane B / 4 on
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          xv[m] = xv[m] + alpha * pv[m];
-          rr2 += rr[m] * rr[m];
-          RR[cell0 + m] = rr[m];
-        }
-        st4(pb.x + gi, xv);
-        st4(rout + gi, rr);
+  for (int u = 0; u < 2; ++u) {
+    TV s0 = (res[2 * u][0] + res[2 * u][1]) + (res[2 * u + 1][0] + res[2 * u + 1][1]);
+    TV s1 = (res[2 * u][2] + res[2 * u][3]) + (res[2 * u + 1][2] + res[2 * u + 1][3]);
+    s0 += __shfl_xor_sync(0xffffffffu, s0, B / 4);
+    s1 += __shfl_xor_sync(0xffffffffu, s1, B / 4);
+    if ((j & 1) == 0) {
+      const int I = i0 >> 1, J = j >> 1, K = (k0 >> 1) + u;
+      const size_t o = (size_t)c * CB * CB * CB + (K * CB + J) * CB + I;
+      r1[o] = s0;
+      r1[o + 1] = s1;
+      if (x1) {  // S r of the next level, where its kernel works cell by cell
+        const TV w4 = TV(0.25) * wl;
+        x1[o] = w4 * (cq.smask ? cq.inv[s3_of<CB>(cq.w3, I, J, K)] : cq.inv[18]) * s0;
+        x1[o + 1] = w4 * (cq.smask ? cq.inv[s3_of<CB>(cq.w3, I + 1, J, K)] : cq.inv[18]) * s1;
       }
     }
-    const int mask = face < 0 ? cs.smask : cs.nbmask[face];
-    const int* w3 = face < 0 ? cs.w3 : cs.nbw3[face];
-    const int kz = cell0 / BB, j = (cell0 / B) % B, i0 = cell0 % B;
-#pragma unroll
-    for (int m = 0; m < 4; ++m)
-      v[m] = w * rr[m] * (mask == 0 ? cs.invtab[18] : cs.invtab[s3_of<B>(w3, i0 + m, j, kz)]);
-  };
-  auto val1 = [&](int f, int n, int cell) {
-    const TV inv = cs.nbmask[f] == 0
-                       ? cs.invtab[18]
-                       : cs.invtab[s3_of<B>(cs.nbw3[f], cell % B, (cell / B) % B, cell / BB)];
-    return w * res((size_t)n * B3 + cell) * inv;
-  };
-  auto valg = [&](int n, int cell) {
-    return w * res((size_t)n * B3 + cell) * inv_diag_any<B, TV>(g, n, cell);
-  };
-  stage_pressure_slab<B, B, NT, TV>(S, cs, g, c, 0, val4, val1, valg, lsh);
-  const TV h = cube_h<TV>(g, g.sp[g.sim[c]], c) * cl;
-  const int i = threadIdx.x % B, j = column_row<B>(threadIdx.x);
-  int o = SL::at(i, j, 1);
-  TV below = S[o - PP], cur = S[o];
-#pragma unroll 4
-  for (int kk = 0; kk < B; ++kk) {
-    const TV above = S[o + PP];
-    TV acc = (cur - S[o - 1]) + (cur - S[o + 1]) + (cur - S[o - SL::P]) +
-             (cur - S[o + SL::P]) + (cur - below) + (cur - above);
-    if (cs.has21) acc = stencil_sum_w<B, TV, B>(S, o, cs, i, j, kk);
-    const int cell = (kk * B + j) * B + i;
-    const size_t gi = (size_t)c * B3 + cell;
-    x[gi] = cur;
-    // FB: RR holds the cell's new residual, stored during the staging
-    RR[cell] = (FB ? RR[cell] : r[gi]) - h * acc;
-    below = cur;
-    cur = above;
-    o += PP;
   }
-  __syncthreads();
-  for (int q = threadIdx.x; q < CB * CB * CB; q += NT) {
-    const int I = q % CB, J = (q / CB) % CB, K = q / (CB * CB);
-    TV sum = TV(0);
+  if constexpr (FB) {  // x last: its loads would hold the registers of another block
+    TV xv[4][4], pv[4][4];
 #pragma unroll
-    for (int d = 0; d < 8; ++d)
-      sum += RR[((2 * K + (d >> 2)) * B + 2 * J + ((d >> 1) & 1)) * B + 2 * I + (d & 1)];
-    r1[(size_t)c * CB * CB * CB + q] = sum;
+    for (int m = 0; m < 4; ++m) {
+      ld4(pb.x + base + m * BB, xv[m]);
+      ld4(pn + base + m * BB, pv[m]);
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      axpy4(alpha, pv[m], xv[m], xv[m]);
+      st4(pb.x + base + m * BB, xv[m]);
+    }
   }
   if constexpr (FB) {
-    double vals[1] = {double(rr2)};
-    block_sum<NT, 1>(vals, red);
-    if (threadIdx.x == 0) acc_add(st, ACC_RR, vals[0]);
+    const TV t[1] = {rr2};
+    double val[1];
+    if constexpr (T::TPC == 32) {
+      TV w = rr2;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+      val[0] = double(w);
+    } else {
+      __shared__ double red[32];
+      block_sum_tv<T::NT, 1, TV>(t, val, red);
+    }
+    if (lt == 0) acc_add_cube(st, ACC_RR, c, val[0]);
   }
 }
 
 template <int B, class TV>
-__global__ __launch_bounds__(B * B) void k_mg_up0_tile(DevGrid g, const TV* __restrict__ ra,
-                                                       const TV* __restrict__ rb,
-                                                       const TV* __restrict__ x,
-                                                       const TV* __restrict__ y1,
-                                                       TV* __restrict__ z, SolveParams prm,
-                                                       int mode, TV wl, TV cl, int finest,
-                                                       int lsh) {
-  cudaGridDependencySynchronize();  // launched after the previous level's kernel
-  using SL = Slab<B, B>;
-  constexpr int NT = B * B, B3 = B * B * B, BB = B * B, PP = SL::P * SL::P, CB = B / 2;
+__global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_up_quad(DevGrid g, const TV* __restrict__ ra,
+                                                          const TV* __restrict__ rb,
+                                                          const TV* __restrict__ y1,
+                                                          TV* __restrict__ z, SolveParams prm,
+                                                          int mode, TV wl, TV cl, int finest,
+                                                          int lsh) {
+  using T = QT<B>;
+  constexpr int B3 = T::B3, BB = T::BB, CB = B / 2, C3 = CB * CB * CB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  TV* S = reinterpret_cast<TV*>(smem_raw);
-  __shared__ CubeSh<TV> cs;
-  __shared__ double red[32];
-  const int c = blockIdx.x, s = g.sim[c];
-  SimState& st = g.ss[s];
-  const bool all = mode == 2;
-  const bool active = all || !st.done;
-  // after a down launch with pass B (rb set) the new residual is in the buffer that
-  // the iteration's parity selects, else in ra
-  const TV* __restrict__ r = (mode == 1 && rb && !(st.iter & 1)) ? rb : ra;
-  double rz = 0.0;
+  __shared__ CubeQ<TV> cqs[T::CPB];
+  const int cub = threadIdx.x / T::TPC, lt = threadIdx.x - cub * T::TPC;
+  const int c = blockIdx.x * T::CPB + cub;
+  TV* S = reinterpret_cast<TV*>(smem_raw) + cub * T::N;
+  TV* gh = S + B3;
+  CubeQ<TV>& cq = cqs[cub];
+  const bool valid = c < g.n_cubes;
+  const CubeLoad L = cube_lookup(g, valid ? c : 0, lt);
+  Halo<B> H;
+  H.lookup(g, valid ? c : 0, lt);
+  cudaGridDependencySynchronize();  // launched after the previous level's kernel
+  poison_tile(reinterpret_cast<TV*>(smem_raw), T::CPB * T::N);
+  SimState& st = g.ss[L.s];
+  const bool active = valid && (mode == 2 || !st.done);
+  TV part[1] = {TV(0)};
   if (active) {
-    load_cube(cs, g, c);
-    __syncthreads();
-    auto xt = [&](int cube, int cell) {
-      const int i = cell % B, j = (cell / B) % B, k = cell / BB;
-      return x[(size_t)cube * B3 + cell] +
-             TV(kMgOver) *
-                 y1[(size_t)cube * CB * CB * CB + ((k >> 1) * CB + (j >> 1)) * CB + (i >> 1)];
+    // after a down launch with pass B (rb set) the new residual is in the buffer that
+    // the iteration's parity selects, else in ra
+    const TV* __restrict__ r = (mode == 1 && rb && !(st.iter & 1)) ? rb : ra;
+    const int pos = lt % T::Q, i0 = (4 * pos) % B, j = (4 * pos) / B, k0 = 4 * (lt / T::Q);
+    const size_t base = (size_t)c * B3 + (k0 * B + j) * B + i0;
+    auto coarse = [&](int cell) {
+      return (((cell / BB) >> 1) * CB + (((cell / B) % B) >> 1)) * CB + ((cell % B) >> 1);
     };
-    auto val4 = [&](int cube, int cell0, int, TV (&v)[4]) {
-      TV xv[4];
-      ld4(x + (size_t)cube * B3 + cell0, xv);
-      const int kz = cell0 / BB, j = (cell0 / B) % B, i0 = cell0 % B;
-      const size_t pb = (size_t)cube * CB * CB * CB + ((kz >> 1) * CB + (j >> 1)) * CB + (i0 >> 1);
-      const TV ya = TV(kMgOver) * y1[pb], yb = TV(kMgOver) * y1[pb + 1];
-      v[0] = xv[0] + ya;
-      v[1] = xv[1] + ya;
-      v[2] = xv[2] + yb;
-      v[3] = xv[3] + yb;
-    };
-    auto val1 = [&](int, int n, int cell) { return xt(n, cell); };
-    auto valg = [&](int n, int cell) { return xt(n, cell); };
-    stage_pressure_slab<B, B, NT, TV>(S, cs, g, c, 0, val4, val1, valg, lsh);
-    const TV h = cube_h<TV>(g, g.sp[s], c) * cl, w = wl;
-    const int i = threadIdx.x % B, j = column_row<B>(threadIdx.x);
-    int o = SL::at(i, j, 1);
-    TV below = S[o - PP], cur = S[o];
-    TV part = TV(0);
-#pragma unroll 4
-    for (int kk = 0; kk < B; ++kk) {
-      const TV above = S[o + PP];
-      TV acc = (cur - S[o - 1]) + (cur - S[o + 1]) + (cur - S[o - SL::P]) +
-               (cur - S[o + SL::P]) + (cur - below) + (cur - above);
-      if (cs.has21) acc = stencil_sum_w<B, TV, B>(S, o, cs, i, j, kk);
-      const size_t gi = (size_t)c * B3 + (kk * B + j) * B + i;
-      const TV inv = cs.smask == 0 ? cs.invtab[18] : cs.invtab[s3_of<B>(cs.w3, i, j, kk)];
-      const TV rv = r[gi];
-      const TV zv = cur + w * inv * (rv - h * acc);
-      z[gi] = zv;
-      part += rv * zv;
-      below = cur;
-      cur = above;
-      o += PP;
+    TV res[4][4], v[4][4], yc[2][2];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) ld4(r + base + m * BB, res[m]);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const TV* y = y1 + (size_t)c * C3 + (((k0 >> 1) + u) * CB + (j >> 1)) * CB + (i0 >> 1);
+      yc[u][0] = y[0];
+      yc[u][1] = y[1];
     }
-    rz = double(part);
+    TV ha[Halo<B>::R][4], hy[Halo<B>::R][2];
+    H.each(lt, [&](int u, int, int n, int cell, int stride) {
+      ldq(r + (size_t)n * B3 + cell, stride, ha[u]);
+      hy[u][0] = y1[(size_t)n * C3 + coarse(cell)];
+      hy[u][1] = y1[(size_t)n * C3 + coarse(cell + 2 * stride)];
+    });
+    cube_publish(cq, g, L, lt);
+    T::sync();
+    const TV over = TV(kMgOver);
+    auto make = [&](int u, int f, int, int cell, int stride, TV (&o)[4]) {
+      TV inv[4];
+      nb_inv<B>(cq, g, c, f, cell, stride, inv);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) o[e] = (wl * inv[e]) * ha[u][e] + over * hy[u][e >> 1];
+    };
+    auto one = [&](int n, int cell) {
+      return wl * inv_diag_any<B, TV>(g, n, cell) * r[(size_t)n * B3 + cell] +
+             over * y1[(size_t)n * C3 + coarse(cell)];
+    };
+    H.store(gh, g, c, lt, make, one, lsh);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      TV inv[4];
+      quad_inv<B>(cq, i0, j, k0 + m, inv);
+      const TV ya = over * yc[m >> 1][0], yb = over * yc[m >> 1][1];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[m][e] = (wl * inv[e]) * res[m][e] + (e < 2 ? ya : yb);
+      own_quad<B>(S, gh, cq, i0, j, k0 + m, v[m]);
+    }
+    T::sync();
+    const TV h = cq.h * cl;
+    quad_column<B>(S, gh, cq, i0, j, k0, v, [&](int m, const TV (&acc)[4]) {
+      TV inv[4], t[4], zv[4];
+      quad_inv<B>(cq, i0, j, k0 + m, inv);
+      axpy4(-h, acc, res[m], t);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) zv[e] = v[m][e] + (wl * inv[e]) * t[e];
+      st4(z + base + m * BB, zv);
+      part[0] += dot4(res[m], zv);
+    });
   }
-  if (all || !finest) return;
-  double vals[1] = {rz};
-  block_sum<NT, 1>(vals, red);
-  if (threadIdx.x == 0 && active) acc_add(st, ACC_RZ, vals[0]);
-  if (last_block(g.counter)) mg_decide(g, prm, mode, NT);
+  if (mode == 2 || !finest) return;
+  double val[1];
+  if constexpr (T::TPC == 32) {
+    TV w = part[0];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+    val[0] = double(w);
+  } else {
+    __shared__ double red[32];
+    block_sum_tv<T::NT, 1, TV>(part, val, red);
+  }
+  if (lt == 0 && active) acc_add_cube(st, ACC_RZ, c, val[0]);
 }
 
-// ---- the aggregate levels, in one block: gather of the cubes' residuals, the V-cycle
-// on the CSR levels k = 0 .. M-1 (k = M-1 the top), result y = ax[0].  The work is a
-// chain of small dependent steps, so it runs from shared memory: with smem_mode 2 the
-// node vectors and the level tables (diagonal, CSR rows, children, parents) are copied
-// in first, all copies in flight at once (cp.async); with 1 only the node vectors live
-// there; with 0 everything stays in the workspace.
-struct TopLevel {
-  double *ar, *ax, *at, *inv;
-  const double *diag, *val;
-  const int *row, *col, *cptr, *cidx, *parent;
+// The decisions of an iteration (mg_decide) after the quad kernels, in a launch of one block:
+// electing a last block in the finest up launch instead keeps every block on its SM for two
+// more round trips to memory.
+__global__ void k_mg_decide(DevGrid g, SolveParams prm, int mode) {
+  cudaGridDependencySynchronize();
+  mg_decide(g, prm, mode, blockDim.x);
+}
+
+// ---- the coarse levels, in one cluster: the per-cube levels from lf on (BL = 4, 2, 1 cells
+// per cube edge), the aggregate levels, and the way back up to level lf, with cluster
+// barriers between the steps.  Each step is a short chain of dependent loads on few cells,
+// so a launch of its own costs more than its work (9 launches, 57 us serialised at 1024
+// cubes); one block of 1024 threads holds the aggregate levels that fit its shared memory
+// (their tables are copied in while the previous kernel drains), the whole cluster the
+// larger ones.  Values that other blocks wrote are read through L2.
+struct AggLevel {
   int n;
+  double *ar, *y, *at, *x;  // residual, result, scratch, S ar (shared memory, or the workspace)
+  const double *diag, *inv, *val;  // K's diagonal, omega / diagonal, -off-diagonals
+  const int *row, *col, *cptr, *cidx, *parent;  // parent: of this level's children
 };
 
-// Shared-memory bytes of the node vectors (3 per node) and of the staged tables: per
-// level the inverse diagonal, the diagonal, the CSR values, rows and columns, and above
-// level 0 the children and parents; every piece 16-byte aligned.
 __host__ __device__ inline size_t top_piece(size_t bytes) { return (bytes + 15) & ~(size_t)15; }
-__host__ __device__ inline size_t top_vec_bytes(const MgDev& mg) {
-  size_t nodes = 0;
-  for (int k = 0; k < mg.M; ++k) nodes += (size_t)mg.n[k];
-  return top_piece(3 * 8 * nodes);
-}
-__host__ __device__ inline size_t top_table_bytes(const MgDev& mg) {
+// shared-memory bytes of aggregate levels k0 .. M-1
+__host__ __device__ inline size_t agg_smem(const MgDev& mg, int n_cubes, int k0) {
   size_t b = 0;
-  for (int k = 0; k < mg.M; ++k) {
-    const size_t n = (size_t)mg.n[k], nnz = (size_t)mg.nnz[k], np = k ? (size_t)mg.n[k - 1] : 0;
-    b += 2 * top_piece(8 * n) + top_piece(8 * nnz) + top_piece(4 * (n + 1)) + top_piece(4 * nnz);
-    if (k) b += top_piece(4 * (n + 1)) + 2 * top_piece(4 * np);
+  for (int k = k0; k < mg.M; ++k) {
+    const size_t n = (size_t)mg.n[k], nnz = (size_t)mg.nnz[k], np = k ? mg.n[k - 1] : n_cubes;
+    b += 6 * top_piece(8 * n) + top_piece(8 * nnz) + top_piece(4 * (n + 1)) + top_piece(4 * nnz);
+    b += top_piece(4 * (n + 1)) + (k ? 2 : 1) * top_piece(4 * np);
   }
   return b;
 }
 
 // asynchronous global -> shared copy of `count` elements of 4 or 8 bytes, by the block
 template <int E>
-__device__ __forceinline__ void copy_async(void* dst, const void* src, int count) {
+__device__ __forceinline__ void copy_async(const void* dst, const void* src, int count) {
   static_assert(E == 4 || E == 8, "element size");
   for (int a = threadIdx.x; a < count; a += blockDim.x) {
-    const unsigned int d = (unsigned int)__cvta_generic_to_shared(static_cast<char*>(dst) + (size_t)E * a);
+    const unsigned int d =
+        (unsigned int)__cvta_generic_to_shared(static_cast<const char*>(dst) + (size_t)E * a);
     const char* s = static_cast<const char*>(src) + (size_t)E * a;
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(d), "l"(s), "n"(E) : "memory");
   }
 }
 
+// The V-cycle on the aggregate levels: W is the set of threads that runs a level (a block on
+// shared memory, or the cluster on the workspace) with its index, size, barrier and loads.
+// An FP64 operation takes a warp 64 cycles here, a barrier of the block about 40, so S ar is
+// formed once per node and not once per edge, and the sums run in few chains.
+struct BlockWorkers {
+  __device__ __forceinline__ int id() const { return threadIdx.x; }
+  __device__ __forceinline__ int count() const { return blockDim.x; }
+  __device__ __forceinline__ void sync() const { __syncthreads(); }
+  __device__ __forceinline__ double ld(const double* p) const { return *p; }
+};
+struct ClusterWorkers {
+  int rank, ranks;
+  __device__ __forceinline__ int id() const { return rank * blockDim.x + threadIdx.x; }
+  __device__ __forceinline__ int count() const { return ranks * blockDim.x; }
+  // the same threads numbered warp by warp over the blocks, so few cells use every SM
+  __device__ __forceinline__ int spread() const {
+    return (((int)threadIdx.x >> 5) * ranks + rank) * 32 + ((int)threadIdx.x & 31);
+  }
+  __device__ __forceinline__ void sync() const { cooperative_groups::this_cluster().sync(); }
+  __device__ __forceinline__ double ld(const double* p) const { return __ldcg(p); }
+};
+// ar - K f on node a, f(b) a node's value: six entries at a time, loaded together, in two
+// chains of additions (64 cycles each)
+template <class W, class F>
+__device__ __forceinline__ double agg_resid(const W& w, const AggLevel& L, int a, double r, const F& f) {
+  double k0 = L.diag[a] * f(a), k1 = 0.0;
+  const int e1 = L.row[a + 1];
+  for (int e = L.row[a]; e < e1; e += 6) {
+    double v[6], x[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const bool in = e + q < e1;
+      v[q] = in ? L.val[e + q] : 0.0;
+      x[q] = in ? f(L.col[e + q]) : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < 6; q += 2) {
+      k0 -= v[q] * x[q];
+      k1 -= v[q + 1] * x[q + 1];
+    }
+  }
+  return r - (k0 + k1);
+}
+template <class W, class V>
+__device__ __forceinline__ double agg_sum(const AggLevel& C, int a, const V& v) {
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  const int e0 = C.cptr[a], e1 = C.cptr[a + 1];
+  for (int e = e0; e < e1; e += 4)
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (e + q < e1) s[q] += v(C.cidx[e + q]);
+  return (s[0] + s[1]) + (s[2] + s[3]);
+}
+// down on level L: x = S ar, at = ar - K x
+template <class W>
+__device__ __forceinline__ void agg_down(const W& w, const AggLevel& L) {
+  for (int a = w.id(); a < L.n; a += w.count()) L.x[a] = L.inv[a] * w.ld(L.ar + a);
+  w.sync();
+  auto xv = [&](int b) { return w.ld(L.x + b); };
+  for (int a = w.id(); a < L.n; a += w.count()) L.at[a] = agg_resid(w, L, a, w.ld(L.ar + a), xv);
+}
+// up on level L: x += s P yc, y = x + S (ar - K x)
+template <class W, class Y>
+__device__ __forceinline__ void agg_up(const W& w, const AggLevel& L, const int* parent, const Y& yc) {
+  for (int a = w.id(); a < L.n; a += w.count()) L.x[a] = w.ld(L.x + a) + kMgOver * yc(parent[a]);
+  w.sync();
+  auto xv = [&](int b) { return w.ld(L.x + b); };
+  for (int a = w.id(); a < L.n; a += w.count())
+    L.y[a] = xv(a) + L.inv[a] * agg_resid(w, L, a, w.ld(L.ar + a), xv);
+}
+// kMgNuTop damped-Jacobi sweeps from zero (the first is S ar); result in y
+template <class W>
+__device__ __forceinline__ void agg_top(const W& w, const AggLevel& L) {
+  double *x = L.at, *o = L.y;
+  static_assert(kMgNuTop == 4, "an odd number of sweeps after the first ends in y");
+  for (int a = w.id(); a < L.n; a += w.count()) x[a] = L.inv[a] * w.ld(L.ar + a);
+  for (int sweep = 1; sweep < kMgNuTop; ++sweep) {
+    w.sync();
+    auto xv = [&](int b) { return w.ld(x + b); };
+    for (int a = w.id(); a < L.n; a += w.count())
+      o[a] = xv(a) + L.inv[a] * agg_resid(w, L, a, w.ld(L.ar + a), xv);
+    double* t = x;
+    x = o;
+    o = t;
+  }
+}
+
+// ---- per-cube levels inside the cluster (the same values as the per-cell kernels; r, x, y
+// of the coarse levels are written and read by different blocks)
+template <int BL, class TV>
+__device__ __forceinline__ void coarse_down(const DevGrid& g, const MgDev& mg, int l, int all,
+                                            const ClusterWorkers& w) {
+  constexpr int B3 = BL * BL * BL, CB = BL > 1 ? BL / 2 : 1, C3 = CB * CB * CB;
+  const TV *r = (const TV*)mg.r[l], *x = (const TV*)mg.x[l];
+  TV* rc = BL > 1 ? (TV*)mg.r[l + 1] : (TV*)mg.rr;
+  TV* xn = BL > 1 ? (TV*)mg.x[l + 1] : nullptr;
+  const TV c4 = TV(1 << (2 * l)), wscale = TV(kMgOmega / double(1 << (2 * l)));
+  const int total = g.n_cubes * B3, rounded = (total + 31) / 32 * 32;
+  for (int t = w.spread(); t < rounded; t += w.count()) {
+    const int c = t / B3, q = t - c * B3, d = BL > 1 ? q & 7 : 0, ci = BL > 1 ? q >> 3 : 0;
+    const bool on = t < total && (all || !g.ss[g.n_sims == 1 ? 0 : g.sim[c]].done);
+    const int I = ci % CB, J = (ci / CB) % CB, K = ci / (CB * CB);
+    TV val = TV(0);
+    if (on) {
+      const int i = BL > 1 ? 2 * I + (d & 1) : 0, j = BL > 1 ? 2 * J + ((d >> 1) & 1) : 0;
+      const int k = BL > 1 ? 2 * K + (d >> 2) : 0;
+      const TV coef = cube_h<TV>(g, g.sp[g.sim[c]], c) * c4;
+      auto xval = [&](int cube, int cell) { return __ldcg(x + (size_t)cube * B3 + cell); };
+      const int cell = lcell<BL>(i, j, k);
+      const TV rv = __ldcg(r + (size_t)c * B3 + cell), xc = xval(c, cell);
+      const TV acc = mg_faces<BL, TV>(g, c, l, i, j, k, xc, xval);
+      val = rv - coef * acc;
+    }
+    if constexpr (BL > 1) {
+      val += __shfl_xor_sync(0xffffffffu, val, 1);
+      val += __shfl_xor_sync(0xffffffffu, val, 2);
+      val += __shfl_xor_sync(0xffffffffu, val, 4);
+    }
+    if (d == 0 && on) {
+      rc[(size_t)c * C3 + ci] = val;
+      if constexpr (BL > 1)
+        xn[(size_t)c * C3 + ci] = next_x<BL, TV>(g, g.sp[g.sim[c]], c, I, J, K, wscale, val);
+    }
+  }
+}
+template <int BL, class TV>
+__device__ __forceinline__ void coarse_up(const DevGrid& g, const MgDev& mg, int l, int all,
+                                          const double* yagg, const ClusterWorkers& w) {
+  constexpr int B3 = BL * BL * BL, CB = BL > 1 ? BL / 2 : 1;
+  const TV *r = (const TV*)mg.r[l], *x = (const TV*)mg.x[l];
+  const TV* yc = BL > 1 ? (const TV*)mg.y[l + 1] : nullptr;
+  TV* y = (TV*)mg.y[l];
+  const int* parent = mg.parent[0];
+  const TV c4 = TV(1 << (2 * l)), wscale = TV(kMgOmega / double(1 << (2 * l)));
+  const int total = g.n_cubes * B3;
+  for (int t = w.spread(); t < total; t += w.count()) {
+    const int c = t / B3, q = t - c * B3;
+    if (!all && g.ss[g.n_sims == 1 ? 0 : g.sim[c]].done) continue;
+    const int i = q % BL, j = (q / BL) % BL, k = q / (BL * BL);
+    const SimParams& sp = g.sp[g.sim[c]];
+    const TV coef = cube_h<TV>(g, sp, c) * c4;
+    auto uval = [&](int cube, int cell) {  // S r + s P y
+      const TV xv = __ldcg(x + (size_t)cube * B3 + cell);
+      if constexpr (BL == 1) {
+        return xv + TV(kMgOver * __ldcg(yagg + parent[cube]));
+      } else {
+        const int a = cell % BL, b = (cell / BL) % BL, e = cell / (BL * BL);
+        return xv + TV(kMgOver) *
+                        __ldcg(yc + (size_t)cube * CB * CB * CB + lcell<CB>(a >> 1, b >> 1, e >> 1));
+      }
+    };
+    const TV xc = uval(c, q);
+    const TV acc = mg_faces<BL, TV>(g, c, l, i, j, k, xc, uval);
+    const TV rv = __ldcg(r + (size_t)c * B3 + q);
+    y[(size_t)c * B3 + q] = xc + smooth_w<BL, TV>(g, sp, c, i, j, k, wscale) * (rv - coef * acc);
+  }
+}
+
+// bl0: cells per cube edge on level lf; levels k < kd of the aggregates run on the cluster.
 template <class TV>
-__device__ void mg_top(const MgDev& mg, const TV* __restrict__ rr, int smem_mode, double* sm) {
-  __shared__ TopLevel lv[kMgMaxM];
+__global__ __launch_bounds__(1024, 1) void k_mg_coarse(DevGrid g, MgDev mg, int lf, int bl0, int kd,
+                                                       int all) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ AggLevel lv[kMgMaxM];
   const int tid = threadIdx.x, NT = blockDim.x;
-  const double w = kMgOmega;
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const ClusterWorkers cw{(int)cl.block_rank(), (int)cl.num_blocks()};
+  const BlockWorkers bw;
+  const bool head = cw.rank == 0;
   if (tid == 0) {  // layout from the sizes alone (no memory reads)
-    int tot = 0;
-    for (int k = 0; k < mg.M; ++k) tot += mg.n[k];
-    int off = 0;
-    unsigned char* base = reinterpret_cast<unsigned char*>(sm);
-    size_t o = top_vec_bytes(mg);
+    unsigned char* o = smem_raw;
     auto take = [&](size_t bytes) {
-      unsigned char* p = base + o;
+      unsigned char* p = o;
       o += top_piece(bytes);
       return p;
     };
     for (int k = 0; k < mg.M; ++k) {
-      TopLevel& L = lv[k];
-      const int n = mg.n[k], nnz = mg.nnz[k], np = k ? mg.n[k - 1] : 0;
-      L.n = n;
-      L.ar = smem_mode ? sm + off : mg.ar[k];
-      L.ax = smem_mode ? sm + tot + off : mg.ax[k];
-      L.at = smem_mode ? sm + 2 * tot + off : mg.at[k];
-      off += n;
-      if (smem_mode == 2) {
-        L.inv = reinterpret_cast<double*>(take(8 * (size_t)n));
-        L.diag = reinterpret_cast<double*>(take(8 * (size_t)n));
-        L.val = reinterpret_cast<double*>(take(8 * (size_t)nnz));
-        L.row = reinterpret_cast<int*>(take(4 * ((size_t)n + 1)));
-        L.col = reinterpret_cast<int*>(take(4 * (size_t)nnz));
-        L.cptr = k ? reinterpret_cast<int*>(take(4 * ((size_t)n + 1))) : mg.cptr[k];
-        L.cidx = k ? reinterpret_cast<int*>(take(4 * (size_t)np)) : mg.cidx[k];
-        L.parent = k ? reinterpret_cast<int*>(take(4 * (size_t)np)) : mg.parent[k];
-      } else {
-        L.inv = nullptr;
-        L.diag = mg.diag[k];
-        L.val = mg.val[k];
-        L.row = mg.row[k];
-        L.col = mg.col[k];
-        L.cptr = mg.cptr[k];
-        L.cidx = mg.cidx[k];
-        L.parent = mg.parent[k];
-      }
+      AggLevel& L = lv[k];
+      const size_t n = mg.n[k], nnz = mg.nnz[k], np = k ? mg.n[k - 1] : g.n_cubes;
+      L = AggLevel{mg.n[k], mg.ar[k], mg.ax[k], mg.at[k], mg.as[k], mg.diag[k], mg.inv[k], mg.val[k],
+                   mg.row[k], mg.col[k], mg.cptr[k], mg.cidx[k], mg.parent[k]};
+      if (k < kd) continue;
+      L.ar = (double*)take(8 * n);
+      L.y = (double*)take(8 * n);
+      L.at = (double*)take(8 * n);
+      L.x = (double*)take(8 * n);
+      L.diag = (double*)take(8 * n);
+      L.inv = (double*)take(8 * n);
+      L.val = (double*)take(8 * nnz);
+      L.row = (int*)take(4 * (n + 1));
+      L.col = (int*)take(4 * nnz);
+      L.cptr = (int*)take(4 * (n + 1));
+      L.cidx = (int*)take(4 * np);
+      if (k) L.parent = (int*)take(4 * np);
     }
   }
   __syncthreads();
-  if (smem_mode == 2) {
-    for (int k = 0; k < mg.M; ++k) {
-      const TopLevel& L = lv[k];
-      const int n = L.n, nnz = mg.nnz[k], np = k ? mg.n[k - 1] : 0;
-      copy_async<8>(const_cast<double*>(L.diag), mg.diag[k], n);
-      copy_async<8>(const_cast<double*>(L.val), mg.val[k], nnz);
-      copy_async<4>(const_cast<int*>(L.row), mg.row[k], n + 1);
-      copy_async<4>(const_cast<int*>(L.col), mg.col[k], nnz);
-      if (k) {
-        copy_async<4>(const_cast<int*>(L.cptr), mg.cptr[k], n + 1);
-        copy_async<4>(const_cast<int*>(L.cidx), mg.cidx[k], np);
-        copy_async<4>(const_cast<int*>(L.parent), mg.parent[k], np);
-      }
+  if (head) {
+    for (int k = kd; k < mg.M; ++k) {
+      const AggLevel& L = lv[k];
+      const int n = L.n, nnz = mg.nnz[k], np = k ? mg.n[k - 1] : g.n_cubes;
+      copy_async<8>(L.diag, mg.diag[k], n);
+      copy_async<8>(L.inv, mg.inv[k], n);
+      copy_async<8>(L.val, mg.val[k], nnz);
+      copy_async<4>(L.row, mg.row[k], n + 1);
+      copy_async<4>(L.col, mg.col[k], nnz);
+      copy_async<4>(L.cptr, mg.cptr[k], n + 1);
+      copy_async<4>(L.cidx, mg.cidx[k], np);
+      if (k) copy_async<4>(L.parent, mg.parent[k], np);
     }
+  }
+  cudaGridDependencySynchronize();  // launched after the previous level's kernel
+  int l = lf, bl = bl0;
+  for (;; ++l, bl >>= 1) {
+    if (bl == 4) coarse_down<4, TV>(g, mg, l, all, cw);
+    else if (bl == 2) coarse_down<2, TV>(g, mg, l, all, cw);
+    else coarse_down<1, TV>(g, mg, l, all, cw);
+    cl.sync();
+    if (bl == 1) break;
+  }
+  if (head) {
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
-    for (int k = 0; k < mg.M; ++k) {
-      const TopLevel& L = lv[k];
-      for (int a = tid; a < L.n; a += NT) {
-        const double d = L.diag[a];
-        L.inv[a] = d > 0.0 ? 1.0 / d : 0.0;
+  }
+  const int top = mg.M - 1;
+  const TV* rr = (const TV*)mg.rr;
+  auto cube_r = [&](int c) { return double(__ldcg(rr + c)); };
+  // down: levels 0 .. kd-1 on the cluster, then the rest in the head block
+  if (kd > 0) {
+    for (int a = cw.id(); a < lv[0].n; a += cw.count()) lv[0].ar[a] = agg_sum<ClusterWorkers>(lv[0], a, cube_r);
+    cl.sync();
+    for (int k = 0; k < kd; ++k) {
+      const AggLevel& L = lv[k];
+      if (k == top) {
+        agg_top(cw, L);
+        cl.sync();
+        break;
+      }
+      agg_down(cw, L);
+      cl.sync();
+      if (k + 1 < kd) {
+        auto child = [&](int c) { return __ldcg(L.at + c); };
+        for (int a = cw.id(); a < lv[k + 1].n; a += cw.count())
+          lv[k + 1].ar[a] = agg_sum<ClusterWorkers>(lv[k + 1], a, child);
+        cl.sync();
       }
     }
   }
-  auto dinv = [&](const TopLevel& L, int a) {
-    if (L.inv) return L.inv[a];
-    const double d = L.diag[a];
-    return d > 0.0 ? 1.0 / d : 0.0;
-  };
-  // at = ar - K ax on level k
-  auto residual = [&](const TopLevel& L) {
-    for (int a = tid; a < L.n; a += NT) {
-      double kx = L.diag[a] * L.ax[a];
-      for (int e = L.row[a]; e < L.row[a + 1]; ++e) kx -= L.val[e] * L.ax[L.col[e]];
-      L.at[a] = L.ar[a] - kx;
-    }
-    __syncthreads();
-  };
-  for (int a = tid; a < mg.n[0]; a += NT) {  // level 0: sums of the cubes' residuals
-    double sum = 0.0;
-    for (int e = mg.cptr[0][a]; e < mg.cptr[0][a + 1]; ++e) sum += double(rr[mg.cidx[0][e]]);
-    lv[0].ar[a] = sum;
-  }
-  __syncthreads();
-  const int top = mg.M - 1;
-  for (int k = 0; k < top; ++k) {
-    const TopLevel& L = lv[k];
-    for (int a = tid; a < L.n; a += NT) L.ax[a] = w * dinv(L, a) * L.ar[a];
-    __syncthreads();
-    residual(L);
-    const TopLevel& C = lv[k + 1];
-    for (int a = tid; a < C.n; a += NT) {
-      double sum = 0.0;
-      for (int e = C.cptr[a]; e < C.cptr[a + 1]; ++e) sum += L.at[C.cidx[e]];
-      C.ar[a] = sum;
-    }
-    __syncthreads();
-  }
-  {
-    const TopLevel& L = lv[top];
-    for (int a = tid; a < L.n; a += NT) L.ax[a] = 0.0;
-    __syncthreads();
-    for (int sweep = 0; sweep < kMgNuTop; ++sweep) {
-      residual(L);
-      for (int a = tid; a < L.n; a += NT) L.ax[a] += w * dinv(L, a) * L.at[a];
+  if (kd <= top) {
+    if (head) {
+      const AggLevel& F = lv[kd];
+      if (kd == 0) {
+        for (int a = tid; a < F.n; a += NT) F.ar[a] = agg_sum<BlockWorkers>(F, a, cube_r);
+      } else {
+        const AggLevel& L = lv[kd - 1];
+        auto child = [&](int c) { return __ldcg(L.at + c); };
+        for (int a = tid; a < F.n; a += NT) F.ar[a] = agg_sum<BlockWorkers>(F, a, child);
+      }
       __syncthreads();
+      for (int k = kd; k < top; ++k) {
+        const AggLevel &L = lv[k], &C = lv[k + 1];
+        agg_down(bw, L);
+        __syncthreads();
+        auto child = [&](int c) { return L.at[c]; };
+        for (int a = tid; a < C.n; a += NT) C.ar[a] = agg_sum<BlockWorkers>(C, a, child);
+        __syncthreads();
+      }
+      agg_top(bw, lv[top]);
+      __syncthreads();
+      for (int k = top - 1; k >= kd; --k) {
+        const AggLevel& C = lv[k + 1];
+        agg_up(bw, lv[k], C.parent, [&](int b) { return C.y[b]; });
+        __syncthreads();
+      }
+      for (int a = tid; a < F.n; a += NT) mg.ax[kd][a] = F.y[a];  // for the other blocks
     }
+    cl.sync();
   }
-  for (int k = top - 1; k >= 0; --k) {
-    const TopLevel& L = lv[k];
-    const TopLevel& C = lv[k + 1];
-    for (int a = tid; a < L.n; a += NT) L.ax[a] += kMgOver * C.ax[C.parent[a]];
-    __syncthreads();
-    residual(L);
-    for (int a = tid; a < L.n; a += NT) L.ax[a] += w * dinv(L, a) * L.at[a];
-    __syncthreads();
+  for (int k = (kd <= top ? kd : top) - 1; k >= 0; --k) {
+    const double* yc = mg.ax[k + 1];
+    agg_up(cw, lv[k], mg.parent[k + 1], [&](int b) { return __ldcg(yc + b); });
+    cl.sync();
   }
-  if (smem_mode) {  // the level-0 result for the up launches
-    for (int a = tid; a < mg.n[0]; a += NT) mg.ax[0][a] = lv[0].ax[a];
+  for (;; --l, bl <<= 1) {
+    if (bl == 4) coarse_up<4, TV>(g, mg, l, all, mg.ax[0], cw);
+    else if (bl == 2) coarse_up<2, TV>(g, mg, l, all, mg.ax[0], cw);
+    else coarse_up<1, TV>(g, mg, l, all, mg.ax[0], cw);
+    if (l == lf) break;
+    cl.sync();
   }
-}
-
-template <class TV>
-__global__ __launch_bounds__(1024) void k_mg_top(MgDev mg, const TV* __restrict__ rr,
-                                                 int smem_mode) {
-  cudaGridDependencySynchronize();  // launched after the previous level's kernel
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  mg_top<TV>(mg, rr, smem_mode, reinterpret_cast<double*>(smem_raw));
 }
 
 // ---------------------------------------------------------------- launcher
 
 template <int BL, class TV>
 static cudaError_t down_t(const Ctx& x, int l, int all) {
-  constexpr int CB = BL > 1 ? BL / 2 : 1;
-  const TV* r = (const TV*)x.mg.r[l];
-  TV* xv = (TV*)x.mg.x[l];
-  TV* rc = BL > 1 ? (TV*)x.mg.r[l + 1] : (TV*)x.mg.rr;
   const double c4 = double(1 << (2 * l));
-  if constexpr (BL > 1) {  // one thread per fine cell
-    const long long n = (long long)x.g.n_cubes * BL * BL * BL;
-    return launch_pdl(k_mg_down_cell<BL, TV>, dim3((unsigned)((n + 255) / 256)), dim3(256), 0,
-                      x.stream, x.g, l, TV(kMgOmega / c4), TV(c4), r, xv, rc, all);
-  } else {
-    const long long n = (long long)x.g.n_cubes * CB * CB * CB;
-    return launch_pdl(k_mg_down<BL, TV>, dim3((unsigned)((n + 255) / 256)), dim3(256), 0,
-                      x.stream, x.g, l, TV(kMgOmega / c4), TV(c4), r, xv, rc, all);
-  }
+  const long long n = (long long)x.g.n_cubes * BL * BL * BL;
+  auto kern = l == 0 ? k_mg_down_cell<BL, TV, false> : k_mg_down_cell<BL, TV, true>;
+  return launch_pdl(kern, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, x.stream, x.g, l,
+                    TV(kMgOmega / c4), TV(c4), (const TV*)x.mg.r[l], (TV*)x.mg.x[l],
+                    (TV*)x.mg.r[l + 1], (TV*)x.mg.x[l + 1], all);
 }
 
 template <int BL, class TV>
 static cudaError_t up_t(const Ctx& x, int l, int all) {
   const long long n = (long long)x.g.n_cubes * BL * BL * BL;
-  const TV* yc = BL > 1 ? (const TV*)x.mg.y[l + 1] : nullptr;
+  const TV* yc = (const TV*)x.mg.y[l + 1];
   const double c4 = double(1 << (2 * l));
   return launch_pdl(k_mg_up<BL, TV>, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, x.stream,
                     x.g, l, TV(kMgOmega / c4), TV(c4), (const TV*)x.mg.r[l], (const TV*)x.mg.x[l],
-                    yc, (const double*)x.mg.ax[0], (const int*)x.mg.parent[0], (TV*)x.mg.y[l],
-                    all);
+                    yc, (TV*)x.mg.y[l], all);
 }
 
 template <class TV>
@@ -807,11 +996,8 @@ static cudaError_t level_t(const Ctx& x, int l, bool down, int all) {
 #define BCM_MG_LEVEL(V) \
   case V: return down ? down_t<V, TV>(x, l, all) : up_t<V, TV>(x, l, all);
   switch (BL) {
-    BCM_MG_LEVEL(16)
-    BCM_MG_LEVEL(8)
     BCM_MG_LEVEL(4)
     BCM_MG_LEVEL(2)
-    BCM_MG_LEVEL(1)
     default: return cudaErrorInvalidValue;
   }
 #undef BCM_MG_LEVEL
@@ -823,14 +1009,13 @@ static cudaError_t up0_t(const Ctx& x, const SolveParams& prm, int mode) {
   const TV* yc = (const TV*)x.mg.y[1];
   return launch_pdl(k_mg_up0<B, NT, TV>, dim3(x.g.n_cubes * (B3 / NT)), dim3(NT), 0, x.stream,
                     x.g, (const TV*)x.mg.r[0], (const TV*)x.mg.x[0], yc,
-                    (const double*)x.mg.ax[0], (const int*)x.mg.parent[0], (TV*)x.mg.y[0], prm,
-                    mode);
+                    (TV*)x.mg.y[0], prm, mode);
 }
 
 template <int B, class TV>
-static cudaError_t down0_tile_t(const Ctx& x, int l, int all, bool fb) {
-  using SL = Slab<B, B>;
-  const size_t sm = sizeof(TV) * ((SL::N + 3) / 4 * 4 + (size_t)B * B * B);
+static cudaError_t down_quad_t(const Ctx& x, int l, int all, bool fb) {
+  using T = QT<B>;
+  const size_t sm = sizeof(TV) * (size_t)T::N * T::CPB;
   PassB<TV> pb{};
   if (fb) {
     pb.x = x.solve64 ? (TV*)x.f.p : (TV*)x.f.e;
@@ -841,72 +1026,99 @@ static cudaError_t down0_tile_t(const Ctx& x, int l, int all, bool fb) {
     pb.rb = (TV*)x.f.s0;
   }
   const double c4 = double(1 << (2 * l));
-  auto kern = fb ? k_mg_down0_tile<B, TV, true> : k_mg_down0_tile<B, TV, false>;
+  auto kern = fb ? k_mg_down_quad<B, TV, true> : k_mg_down_quad<B, TV, false>;
   cudaError_t e = allow_dynamic_smem(kern, sm);
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(x.g.n_cubes), dim3(B * B), sm, x.stream, x.g,
-                    (const TV*)x.mg.r[l], (TV*)x.mg.x[l], (TV*)x.mg.r[l + 1], all, pb,
-                    TV(kMgOmega / c4), TV(c4), l);
+  return launch_pdl(kern, dim3((x.g.n_cubes + T::CPB - 1) / T::CPB), dim3(T::NT), sm, x.stream, x.g,
+                    (const TV*)x.mg.r[l], (TV*)x.mg.r[l + 1],
+                    B / 2 <= 4 ? (TV*)x.mg.x[l + 1] : (TV*)nullptr, all, pb, TV(kMgOmega / c4),
+                    TV(c4), l);
 }
 
 template <int B, class TV>
-static cudaError_t up0_tile_t(const Ctx& x, int l, const SolveParams& prm, int mode, bool fb) {
-  using SL = Slab<B, B>;
-  const size_t sm = sizeof(TV) * SL::N;
+static cudaError_t up_quad_t(const Ctx& x, int l, const SolveParams& prm, int mode, bool fb) {
+  using T = QT<B>;
+  const size_t sm = sizeof(TV) * (size_t)T::N * T::CPB;
   const double c4 = double(1 << (2 * l));
-  auto kern = k_mg_up0_tile<B, TV>;
+  auto kern = k_mg_up_quad<B, TV>;
   cudaError_t e = allow_dynamic_smem(kern, sm);
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(x.g.n_cubes), dim3(B * B), sm, x.stream, x.g,
+  return launch_pdl(kern, dim3((x.g.n_cubes + T::CPB - 1) / T::CPB), dim3(T::NT), sm, x.stream, x.g,
                     (const TV*)x.mg.r[l], fb ? (const TV*)x.f.s0 : (const TV*)nullptr,
-                    (const TV*)x.mg.x[l], (const TV*)x.mg.y[l + 1], (TV*)x.mg.y[l], prm, mode,
-                    TV(kMgOmega / c4), TV(c4), l == 0 ? 1 : 0, l);
+                    (const TV*)x.mg.y[l + 1], (TV*)x.mg.y[l], prm, mode, TV(kMgOmega / c4), TV(c4),
+                    l == 0 ? 1 : 0, l);
+}
+
+// First level of the coarse kernel: at most 4^3 cells per cube, and no more cells than the
+// largest cluster has threads (a launch over all SMs does more of them faster).
+static int coarse_from(const Ctx& x) {
+  int l = 1;
+  while (l < x.mg.L && ((x.B >> l) > 4 || (long long)x.g.n_cubes * (x.B >> l) * (x.B >> l) * (x.B >> l) >
+                                              16LL * 1024))
+    ++l;
+  return l;
+}
+template <class TV>
+static cudaError_t coarse_t(const Ctx& x, int lf, int all) {
+  // aggregate levels of more than 1024 nodes, or that do not fit, run on the cluster
+  int kd = 0;
+  while (kd < x.mg.M && (x.mg.n[kd] > 1024 || agg_smem(x.mg, x.g.n_cubes, kd) > 200 * 1024)) ++kd;
+  const size_t sm = agg_smem(x.mg, x.g.n_cubes, kd);
+  const long long bl = x.B >> lf, cells = x.g.n_cubes * bl * bl * bl;
+  int ranks = 1;  // a cell per thread, up to the largest cluster
+  while (ranks < 16 && (cells > 1024LL * ranks || (kd > 0 && x.mg.n[0] > 1024 * ranks))) ranks *= 2;
+  auto kern = k_mg_coarse<TV>;
+  cudaError_t e = allow_dynamic_smem(kern, sm);
+  if (e != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
+    return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(ranks);
+  cfg.blockDim = dim3(1024);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = x.stream;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ranks;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kern, x.g, x.mg, lf, (int)bl, kd, all);
 }
 
 template <class TV>
 static cudaError_t vcycle_t(const Ctx& x, const SolveParams& prm, int mode) {
   const int all = mode == 2 ? 1 : 0;
   cudaError_t e;
-  // the finest level of 8^3 and 16^3 cubes through the shared-memory tile, which after
+  // the finest level of 8^3 and 16^3 cubes through the quad tile, which after
   // pass A also does the PCG's pass B; other cube sizes launch pass B first
   const bool tile = x.B == 8 || x.B == 16;
   const bool fb = tile && mode == 1;
   if (mode == 1 && !fb && (e = launch_cg_b(x, prm)) != cudaSuccess) return e;
-  e = tile ? (x.B == 16 ? down0_tile_t<16, TV>(x, 0, all, fb) : down0_tile_t<8, TV>(x, 0, all, fb))
+  e = tile ? (x.B == 16 ? down_quad_t<16, TV>(x, 0, all, fb) : down_quad_t<8, TV>(x, 0, all, fb))
            : level_t<TV>(x, 0, true, all);
   if (e != cudaSuccess) return e;
-  // levels of 8^3 cells per cube through the tile too, the smaller ones per cell
-  for (int l = 1; l <= x.mg.L; ++l)
-    if ((e = (x.B >> l) == 8 ? down0_tile_t<8, TV>(x, l, all, false)
+  // levels of 8^3 cells per cube through the quad tile too, the smaller ones per cell down
+  // to the level the coarse kernel takes over
+  const int lf = coarse_from(x);
+  for (int l = 1; l < lf; ++l)
+    if ((e = (x.B >> l) == 8 ? down_quad_t<8, TV>(x, l, all, false)
                              : level_t<TV>(x, l, true, all)) != cudaSuccess)
       return e;
-  {
-    // node vectors and, where they fit, the level tables in shared memory
-    const size_t vec = top_vec_bytes(x.mg), tables = top_table_bytes(x.mg);
-    const int smem_mode = vec + tables <= 200 * 1024 ? 2 : vec <= 160 * 1024 ? 1 : 0;
-    const size_t sm = smem_mode == 2 ? vec + tables : smem_mode == 1 ? vec : 0;
-    int maxn = 0;
-    for (int k = 0; k < x.mg.M; ++k) maxn = x.mg.n[k] > maxn ? x.mg.n[k] : maxn;
-    const int nt = maxn < 64 ? 64 : maxn > 1024 ? 1024 : (maxn + 31) / 32 * 32;
-    auto kern = k_mg_top<TV>;
-    if (smem_mode && (e = allow_dynamic_smem(kern, sm)) != cudaSuccess) return e;
-    if ((e = launch_pdl(kern, dim3(1), dim3(nt), sm, x.stream, x.mg, (const TV*)x.mg.rr,
-                        smem_mode)) != cudaSuccess)
-      return e;
-  }
-  for (int l = x.mg.L; l >= 1; --l)
-    if ((e = (x.B >> l) == 8 ? up0_tile_t<8, TV>(x, l, prm, mode, false)
+  if ((e = coarse_t<TV>(x, lf, all)) != cudaSuccess) return e;
+  for (int l = lf - 1; l >= 1; --l)
+    if ((e = (x.B >> l) == 8 ? up_quad_t<8, TV>(x, l, prm, mode, false)
                              : level_t<TV>(x, l, false, all)) != cudaSuccess)
       return e;
-  if (tile)
-    return x.B == 16 ? up0_tile_t<16, TV>(x, 0, prm, mode, fb)
-                     : up0_tile_t<8, TV>(x, 0, prm, mode, fb);
-  switch (x.B) {
-    case 4: return up0_t<4, TV>(x, prm, mode);
-    case 8: return up0_t<8, TV>(x, prm, mode);
-    case 16: return up0_t<16, TV>(x, prm, mode);
-    default: return cudaErrorInvalidValue;
+  if (tile) {
+    e = x.B == 16 ? up_quad_t<16, TV>(x, 0, prm, mode, fb) : up_quad_t<8, TV>(x, 0, prm, mode, fb);
+    if (e != cudaSuccess || mode == 2) return e;
+    return launch_pdl(k_mg_decide, dim3(1), dim3(x.g.n_sims > 256 ? 256 : (x.g.n_sims + 31) / 32 * 32),
+                      0, x.stream, x.g, prm, mode);
   }
+  return x.B == 4 ? up0_t<4, TV>(x, prm, mode) : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_mg_vcycle(const Ctx& x, const SolveParams& prm, int mode) {

@@ -21,7 +21,7 @@
 // the number of the iteration it belongs to, and a warp of every block that holds cells
 // of the sim reads the words of that sim's blocks until all carry the iteration's number:
 // the sum and the barrier are one message each way, sims do not wait for one another,
-// and the summation order is fixed (the same result on every run).  The waits end at
+// and the order of the additions within a solve is fixed.  The waits end at
 // barrier_timeout_ns (BCM_E_TIMEOUT).
 //
 // What bounds it: the two exchanges on small grids (2.2k cycles among 16 blocks, 3.1k
@@ -43,6 +43,7 @@
 #include "bcm_internal.cuh"
 #include "bcm_kernels.h"
 #include "bcm_persist.cuh"
+#include "bcm_quad.cuh"
 
 namespace bcm {
 
@@ -82,27 +83,6 @@ __device__ __forceinline__ unsigned long long word_get(const Word* w, double& v)
 // After the words of a wait: the other blocks' writes before their words are visible.
 // (Acquire loads in the wait's loop instead would run one after another.)
 __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
-
-// 1 / d by Newton's iteration y <- y + y (1 - d y) from the hardware's approximate
-// reciprocal (23 bits): two steps, or one (46 bits) where the quotient is then rounded to
-// FP32.  An FP64 operation takes 64 cycles on this part and the compiler's division
-// 1460; these take about 450 and 250, twice per iteration of the solver.  Exponents near
-// the ends of the range go to the division.
-template <class TV>
-__device__ __forceinline__ double quick_rcp(double d) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-  const unsigned ex = (unsigned)__double2hiint(y) >> 20 & 0x7ffu;
-  if (ex - 64u > 1920u) return 1.0 / d;
-  y = fma(y, fma(-d, y, 1.0), y);
-  return sizeof(TV) == 8 ? fma(y, fma(-d, y, 1.0), y) : y;
-}
-template <class TV>
-__device__ __forceinline__ double quick_div(double a, double d, double y) {  // y = 1 / d
-  double q = a * y;
-  if (sizeof(TV) == 8) q = fma(fma(-d, q, a), y, q);
-  return isfinite(q) ? q : a / d;
-}
 
 // Shape of a launch, chosen on the host (res_shape).
 struct ResShape {
@@ -294,83 +274,6 @@ __device__ __forceinline__ void ldcg4(const double* p, double (&v)[4]) {
   const double2 a = __ldcg(reinterpret_cast<const double2*>(p));
   const double2 b = __ldcg(reinterpret_cast<const double2*>(p) + 1);
   v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
-}
-
-// Quads of cells in FP32 as two packed pairs (one instruction per pair), in FP64 plain.
-__device__ __forceinline__ unsigned long long pk(float a, float b) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void upk(unsigned long long r, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
-}
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
-  unsigned long long r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ unsigned long long sub2(unsigned long long a, unsigned long long b) {
-  unsigned long long r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b,
-                                                   unsigned long long c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-// out = a x + y
-__device__ __forceinline__ void axpy4(float a, const float (&x)[4], const float (&y)[4],
-                                      float (&out)[4]) {
-  const unsigned long long aa = pk(a, a);
-  const unsigned long long l = fma2(aa, pk(x[0], x[1]), pk(y[0], y[1]));
-  const unsigned long long h = fma2(aa, pk(x[2], x[3]), pk(y[2], y[3]));
-  upk(l, out[0], out[1]);
-  upk(h, out[2], out[3]);
-}
-__device__ __forceinline__ void axpy4(double a, const double (&x)[4], const double (&y)[4],
-                                      double (&out)[4]) {
-#pragma unroll
-  for (int e = 0; e < 4; ++e) out[e] = fma(a, x[e], y[e]);
-}
-__device__ __forceinline__ float dot4(const float (&x)[4], const float (&y)[4]) {
-  float a, b;
-  upk(fma2(pk(x[2], x[3]), pk(y[2], y[3]), fma2(pk(x[0], x[1]), pk(y[0], y[1]), 0ull)), a, b);
-  return a + b;
-}
-__device__ __forceinline__ double dot4(const double (&x)[4], const double (&y)[4]) {
-  return fma(x[3], y[3], fma(x[2], y[2], fma(x[1], y[1], x[0] * y[0])));
-}
-// K p / h of a quad: its cells, the cells before and after it along x, the quads across y
-// and z.  FP64: six operations a cell; FP32 sums the differences, which are exact for
-// close values.
-__device__ __forceinline__ void seven_point(const double (&c)[4], double xl, double xh,
-                                            const double (&ym)[4], const double (&yp)[4],
-                                            const double (&zm)[4], const double (&zp)[4],
-                                            double (&acc)[4]) {
-  const double xm[4] = {xl, c[0], c[1], c[2]}, xp[4] = {c[1], c[2], c[3], xh};
-#pragma unroll
-  for (int e = 0; e < 4; ++e)
-    acc[e] = fma(6.0, c[e], -(((xm[e] + xp[e]) + (ym[e] + yp[e])) + (zm[e] + zp[e])));
-}
-__device__ __forceinline__ void seven_point(const float (&c)[4], float xl, float xh,
-                                            const float (&ym)[4], const float (&yp)[4],
-                                            const float (&zm)[4], const float (&zp)[4],
-                                            float (&acc)[4]) {
-  const float d01 = c[0] - c[1], d12 = c[1] - c[2], d23 = c[2] - c[3];
-  const float x[4] = {(c[0] - xl) + d01, d12 - d01, d23 - d12, (c[3] - xh) - d23};
-#pragma unroll
-  for (int u = 0; u < 4; u += 2) {
-    const unsigned long long cc = pk(c[u], c[u + 1]);
-    unsigned long long a = pk(x[u], x[u + 1]);
-    a = add2(a, sub2(cc, pk(ym[u], ym[u + 1])));
-    a = add2(a, sub2(cc, pk(yp[u], yp[u + 1])));
-    a = add2(a, sub2(cc, pk(zm[u], zm[u + 1])));
-    a = add2(a, sub2(cc, pk(zp[u], zp[u + 1])));
-    upk(a, acc[u], acc[u + 1]);
-  }
 }
 
 // ---------------------------------------------------------------- the kernel

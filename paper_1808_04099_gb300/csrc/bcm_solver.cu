@@ -19,6 +19,7 @@
 #include "bcm_internal.cuh"
 #include "bcm_kernels.h"
 #include "bcm_persist.cuh"
+#include "bcm_quad.cuh"
 
 namespace bcm {
 
@@ -172,6 +173,20 @@ __global__ __launch_bounds__(NT) void k_residual(DevGrid g, const double* __rest
   }
 }
 
+// alpha of every running sim from the completed <p, K p> (last block of pass A)
+__device__ __forceinline__ void cg_alpha(const DevGrid& g, int nt) {
+  for (int qq = threadIdx.x; qq < g.n_sims; qq += nt) {
+    SimState& t = g.ss[qq];
+    const double pqs = acc_take(t, ACC_PQ);
+    if (t.done) continue;
+    t.alpha = (pqs != 0.0) ? t.rz / pqs : 0.0;
+    if (!isfinite(pqs)) {
+      t.nonfinite = 1;
+      t.alpha = 0.0;
+    }
+  }
+}
+
 // ===========================================================================
 // PCG pass A on a z-slab of KS planes of one cube:
 //   p_new = z + beta p_old (z = r / diag), q = K p_new, <p_new, q>.
@@ -254,18 +269,111 @@ __global__ __launch_bounds__(NT) void k_cg_a(DevGrid g, const TV* __restrict__ r
   double vals[1];
   block_sum_tv<NT, 1, TV>(pp, vals, red);
   if (threadIdx.x == 0 && active) acc_add(st, ACC_PQ, vals[0]);
-  if (last_block(g.counter)) {
-    for (int qq = threadIdx.x; qq < g.n_sims; qq += NT) {
-      SimState& t = g.ss[qq];
-      const double pqs = acc_take(t, ACC_PQ);
-      if (t.done) continue;
-      t.alpha = (pqs != 0.0) ? t.rz / pqs : 0.0;
-      if (!isfinite(pqs)) {
-        t.nonfinite = 1;
-        t.alpha = 0.0;
-      }
+  if (last_block(g.counter)) cg_alpha(g, NT);
+}
+
+// ===========================================================================
+// PCG pass A on whole cubes of 16^3 or 8^3 by quad tiles (bcm_quad.cuh); Z: z = M^-1 r
+// comes from the multigrid V-cycle, else it is r / diag.
+// ===========================================================================
+template <int B, class TV, bool Z>
+__global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_cg_a_quad(DevGrid g, const TV* __restrict__ r,
+                                                         TV* __restrict__ p0, TV* __restrict__ p1,
+                                                         TV* __restrict__ q) {
+  using T = QT<B>;
+  constexpr int B3 = T::B3, BB = T::BB;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ CubeQ<TV> cqs[T::CPB];
+  const int cub = threadIdx.x / T::TPC, lt = threadIdx.x - cub * T::TPC;
+  const int c = blockIdx.x * T::CPB + cub;
+  TV* S = reinterpret_cast<TV*>(smem_raw) + cub * T::N;
+  TV* gh = S + B3;
+  CubeQ<TV>& cq = cqs[cub];
+  const bool valid = c < g.n_cubes;
+  const CubeLoad L = cube_lookup(g, valid ? c : 0, lt);
+  Halo<B> H;
+  H.lookup(g, valid ? c : 0, lt);
+  cudaGridDependencySynchronize();  // (multigrid iteration: launched while the V-cycle drains)
+  poison_tile(reinterpret_cast<TV*>(smem_raw), T::CPB * T::N);
+  SimState& st = g.ss[L.s];
+  const bool active = valid && !st.done;
+  TV part[1] = {TV(0)};
+  if (active) {
+    const int it = st.iter;
+    const TV* __restrict__ pold = (it & 1) ? p1 : p0;
+    TV* __restrict__ pnew = (it & 1) ? p0 : p1;
+    const TV beta = TV(st.beta);
+    const bool first = it == 0;
+    const int pos = lt % T::Q, i0 = (4 * pos) % B, j = (4 * pos) / B, k0 = 4 * (lt / T::Q);
+    const size_t base = (size_t)c * B3 + (k0 * B + j) * B + i0;
+    TV v[4][4], pp[4][4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      ld4(r + base + m * BB, v[m]);
+      if (!first) ld4(pold + base + m * BB, pp[m]);
     }
+    TV ha[Halo<B>::R][4], hb[Halo<B>::R][4];
+    H.each(lt, [&](int u, int, int n, int cell, int stride) {
+      const size_t gi = (size_t)n * B3 + cell;
+      ldq(r + gi, stride, ha[u]);
+      if (!first) ldq(pold + gi, stride, hb[u]);
+    });
+    cube_publish(cq, g, L, lt);
+    T::sync();
+    auto make = [&](int u, int f, int, int cell, int stride, TV (&o)[4]) {
+      if constexpr (!Z) {
+        TV inv[4];
+        nb_inv<B>(cq, g, c, f, cell, stride, inv);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) ha[u][e] *= inv[e];
+      }
+      if (!first) axpy4(beta, hb[u], ha[u], o);
+      else
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[e] = ha[u][e];
+    };
+    auto one = [&](int n, int cell) {
+      const size_t gi = (size_t)n * B3 + cell;
+      TV z = r[gi];
+      if constexpr (!Z) z *= inv_diag_any<B, TV>(g, n, cell);
+      return first ? z : z + beta * pold[gi];
+    };
+    H.store(gh, g, c, lt, make, one, 0);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      if constexpr (!Z) {
+        TV inv[4];
+        quad_inv<B>(cq, i0, j, k0 + m, inv);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[m][e] *= inv[e];
+      }
+      if (!first) axpy4(beta, pp[m], v[m], v[m]);
+      own_quad<B>(S, gh, cq, i0, j, k0 + m, v[m]);
+      st4(pnew + base + m * BB, v[m]);
+    }
+    T::sync();
+    const TV h = cq.h;
+    quad_column<B>(S, gh, cq, i0, j, k0, v, [&](int m, const TV (&acc)[4]) {
+      TV qv[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) qv[e] = h * acc[e];
+      st4(q + base + m * BB, qv);
+      part[0] += dot4(v[m], qv);
+    });
   }
+  double val[1];
+  if constexpr (T::TPC == 32) {
+    TV w = part[0];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+    val[0] = double(w);
+  } else {
+    __shared__ double red[32];
+    block_sum_tv<T::NT, 1, TV>(part, val, red);
+  }
+  if (lt == 0 && active) acc_add_cube(st, ACC_PQ, c, val[0]);
+  // with the multigrid the down launch that follows forms alpha from the sums itself
+  if (!Z && last_block(g.counter)) cg_alpha(g, T::NT);
 }
 
 // ===========================================================================
@@ -560,10 +668,27 @@ cudaError_t launch_residual(const Ctx& x, const SolveParams& prm) {
     default: return cudaErrorInvalidValue;                   \
   }
 
+template <int B, class TV>
+static cudaError_t cg_a_quad_t(const Ctx& x, const SolveParams& prm) {
+  using T = QT<B>;
+  const size_t sm = sizeof(TV) * (size_t)T::N * T::CPB;
+  auto kern = prm.mg ? k_cg_a_quad<B, TV, true> : k_cg_a_quad<B, TV, false>;
+  cudaError_t e = allow_dynamic_smem(kern, sm);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(kern, dim3((x.g.n_cubes + T::CPB - 1) / T::CPB), dim3(T::NT), sm, x.stream, x.g,
+                    prm.mg ? (const TV*)x.mg.y[0] : (const TV*)x.f.r, (TV*)x.f.p0, (TV*)x.f.p1,
+                    (TV*)x.f.q);
+}
 template <class TV>
 static cudaError_t cg_a_t(const Ctx& x, const SolveParams& prm) {
+  // whole cubes of 16^3 and 8^3 by quad tiles; slabs of them and cubes of 4^3 by padded ones
+  // (the multigrid's down launch expects the sums as the quad kernel leaves them)
+  if ((x.slabs_a == 1 || prm.mg) && x.B == 16) return cg_a_quad_t<16, TV>(x, prm);
+  if ((x.slabs_a == 1 || prm.mg) && x.B == 8) return cg_a_quad_t<8, TV>(x, prm);
   BCM_DISPATCH_B(x.B, {
     BCM_DISPATCH_KS(x.slabs_a, {
+      if constexpr (KS == B && B != 4) return cudaErrorInvalidValue;  // quad tiles, above
+      else {
       constexpr int NT = threads_for<B>();
       const size_t sm = sizeof(TV) * Slab<B, KS>::N;
       auto ka = k_cg_a<B, KS, NT, TV>;
@@ -578,6 +703,7 @@ static cudaError_t cg_a_t(const Ctx& x, const SolveParams& prm) {
         ka<<<x.g.n_cubes * (B / KS), NT, sm, x.stream>>>(x.g, (const TV*)x.f.r, zv,
                                                          (TV*)x.f.p0, (TV*)x.f.p1, (TV*)x.f.q,
                                                          prm);
+      }
       }
     });
   });
