@@ -50,40 +50,97 @@ __device__ __forceinline__ int line_at(int d, int a, int b, int pos) {
   return d == 0 ? tix<B>(pos, a, b) : (d == 1 ? tix<B>(a, pos, b) : tix<B>(a, b, pos));
 }
 
-template <int B>
-__device__ void lift_forward(double* X, int d, int a, int b, int m) {
-  double tmp[B];
-  const int h = m / 2;
-  for (int i = 0; i < h; ++i) {
-    const double x0 = X[line_at<B>(d, a, b, 2 * i)];
-    const double right = (2 * i + 2 < m) ? X[line_at<B>(d, a, b, 2 * i + 2)] : x0;
-    const double t = __dmul_rn(0.5, __dadd_rn(x0, right));
-    tmp[h + i] = __dsub_rn(X[line_at<B>(d, a, b, 2 * i + 1)], t);
+// One line of M values of a lifting pass, in registers (M at compile time: a line held in
+// an array of run-time length lives in local memory).  The halves and quarters are exact,
+// so x - (p + q) / 2 as one fused operation rounds as the separate product and difference
+// do, and at the ends (p + p) / 2 is p: 2 FP64 operations a value instead of 3 (the passes
+// are bound by the FP64 pipe: on 4.2M cells the forward kernel takes 100 us, 191 with the
+// divisions of the quantizer and run-time lines; decoding 150 us, 165 before).
+template <int B, int M>
+__device__ __forceinline__ void lift_forward(double* X, int d, int a, int b) {
+  constexpr int H = M / 2;
+  double x[M], dt[H];
+#pragma unroll
+  for (int i = 0; i < M; ++i) x[i] = X[line_at<B>(d, a, b, i)];
+#pragma unroll
+  for (int i = 0; i < H; ++i)
+    dt[i] = i + 1 < H ? __fma_rn(-0.5, __dadd_rn(x[2 * i], x[i + 1 < H ? 2 * i + 2 : 0]), x[2 * i + 1])
+                      : __dsub_rn(x[2 * i + 1], x[2 * i]);
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    X[line_at<B>(d, a, b, i)] = i > 0 ? __fma_rn(0.25, __dadd_rn(dt[i > 0 ? i - 1 : 0], dt[i]), x[2 * i])
+                                      : __fma_rn(0.5, dt[0], x[0]);
+    X[line_at<B>(d, a, b, H + i)] = dt[i];
   }
-  for (int i = 0; i < h; ++i) {
-    const double dl = i > 0 ? tmp[h + i - 1] : tmp[h];
-    const double t = __dmul_rn(0.25, __dadd_rn(dl, tmp[h + i]));
-    tmp[i] = __dadd_rn(X[line_at<B>(d, a, b, 2 * i)], t);
-  }
-  for (int i = 0; i < m; ++i) X[line_at<B>(d, a, b, i)] = tmp[i];
 }
 
-template <int B>
-__device__ void lift_inverse(double* X, int d, int a, int b, int m) {
-  double tmp[B];
-  const int h = m / 2;
-  for (int i = 0; i < h; ++i) {
-    const double dl = i > 0 ? X[line_at<B>(d, a, b, h + i - 1)] : X[line_at<B>(d, a, b, h)];
-    const double t = __dmul_rn(0.25, __dadd_rn(dl, X[line_at<B>(d, a, b, h + i)]));
-    tmp[2 * i] = __dsub_rn(X[line_at<B>(d, a, b, i)], t);
+template <int B, int M>
+__device__ __forceinline__ void lift_inverse(double* X, int d, int a, int b) {
+  constexpr int H = M / 2;
+  double e[H], dt[H];
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    e[i] = X[line_at<B>(d, a, b, i)];
+    dt[i] = X[line_at<B>(d, a, b, H + i)];
   }
-  for (int i = 0; i < h; ++i) {
-    const double right = (2 * i + 2 < m) ? tmp[2 * i + 2] : tmp[2 * i];
-    const double t = __dmul_rn(0.5, __dadd_rn(tmp[2 * i], right));
-    tmp[2 * i + 1] = __dadd_rn(X[line_at<B>(d, a, b, h + i)], t);
+#pragma unroll
+  for (int i = 0; i < H; ++i)
+    e[i] = i > 0 ? __fma_rn(-0.25, __dadd_rn(dt[i > 0 ? i - 1 : 0], dt[i]), e[i])
+                 : __fma_rn(-0.5, dt[0], e[0]);
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    X[line_at<B>(d, a, b, 2 * i)] = e[i];
+    X[line_at<B>(d, a, b, 2 * i + 1)] =
+        i + 1 < H ? __fma_rn(0.5, __dadd_rn(e[i], e[i + 1 < H ? i + 1 : 0]), dt[i])
+                  : __dadd_rn(dt[i], e[i]);
   }
-  for (int i = 0; i < m; ++i) X[line_at<B>(d, a, b, i)] = tmp[i];
 }
+
+// the levels M = B, B/2, ..., 2 forward, and back
+template <int B, int M>
+__device__ __forceinline__ void wav_forward(double* X) {
+  if constexpr (M >= 2) {
+#pragma unroll 1
+    for (int d = 0; d < 3; ++d) {
+      if (threadIdx.x < M * M) lift_forward<B, M>(X, d, threadIdx.x % M, threadIdx.x / M);
+      __syncthreads();
+    }
+    wav_forward<B, M / 2>(X);
+  }
+}
+template <int B, int M>
+__device__ __forceinline__ void wav_inverse(double* X) {
+  if constexpr (M >= 2) {
+    wav_inverse<B, M / 2>(X);
+#pragma unroll 1
+    for (int d = 2; d >= 0; --d) {
+      if (threadIdx.x < M * M) lift_inverse<B, M>(X, d, threadIdx.x % M, threadIdx.x / M);
+      __syncthreads();
+    }
+  }
+}
+
+// rint(c / step) as an integer, |result| < 2^30, or *bad.  With y = 1 / step rounded,
+// t = c y is within 2^-51 |t| of the rounded quotient, so below 2^29 both round to the same
+// integer unless t lies within 2^-20 of a half-integer; only then, and when y is not
+// finite (wav_inv), the quotient itself is formed (a division costs about 20 FP64
+// operations, this 4: adding 3 2^51 leaves the rounded integer in the low word).
+__device__ __forceinline__ int32_t quantize(double c, double step, double y, bool* bad) {
+  constexpr double kMagic52 = 6755399441055744.0;
+  const double t = __dmul_rn(c, y), m = __dadd_rn(t, kMagic52);
+  const double off = __dsub_rn(t, __dsub_rn(m, kMagic52));
+  const int ht = __double2hiint(t) & 0x7fffffff, ho = __double2hiint(off) & 0x7fffffff;
+  // 0x41c00000: 2^29; 0x3fdffff8: 0.5 - 2^-20
+  if (ht < 0x41c00000 && ho < 0x3fdffff8) return __double2loint(m);
+  const double r = rint(__ddiv_rn(c, step));
+  if (!(fabs(r) < 1073741824.0)) {
+    *bad = true;
+    return 0;
+  }
+  return (int32_t)r;
+}
+// 1 / step for quantize, NaN (every value takes the quotient) near the ends of the range
+inline double wav_inv(double step) { return step > 1e-280 && step < 1e280 ? 1.0 / step : NAN; }
 
 __device__ __forceinline__ uint32_t zigzag(int32_t q) {
   return ((uint32_t)q << 1) ^ (uint32_t)(q >> 31);
@@ -116,6 +173,7 @@ __device__ __forceinline__ unsigned long long block_sum_u64(unsigned long long v
 // forward transform, quantization, Rice parameter and record size of one cube
 template <int B, class T>
 __global__ __launch_bounds__(B * B) void k_wav_forward(const T* __restrict__ f, double step,
+                                                       double inv,
                                                        uint32_t* __restrict__ zc,
                                                        uint32_t* __restrict__ cube_nbits,
                                                        uint32_t* __restrict__ cube_k,
@@ -128,27 +186,24 @@ __global__ __launch_bounds__(B * B) void k_wav_forward(const T* __restrict__ f, 
   for (int q = threadIdx.x; q < B3; q += NT)
     X[tix<B>(q % B, (q / B) % B, q / (B * B))] = double(f[(size_t)c * B3 + q]);
   __syncthreads();
-  for (int m = B; m >= 2; m /= 2)
-    for (int d = 0; d < 3; ++d) {
-      if (threadIdx.x < m * m) lift_forward<B>(X, d, threadIdx.x % m, threadIdx.x / m, m);
-      __syncthreads();
-    }
+  wav_forward<B, B>(X);
   unsigned long long zsum = 0;
-  for (int q = threadIdx.x; q < B3; q += NT) {
-    double r = rint(__ddiv_rn(X[tix<B>(q % B, (q / B) % B, q / (B * B))], step));
-    if (!(fabs(r) < 1073741824.0)) {
-      atomicOr(err, 1);
-      r = 0.0;
-    }
-    const uint32_t z = zigzag((int32_t)r);
-    zc[(size_t)c * B3 + q] = z;
-    zsum += z;
+  bool bad = false;
+  uint32_t zq[B3 / NT];
+#pragma unroll
+  for (int u = 0; u < B3 / NT; ++u) {
+    const int q = threadIdx.x + u * NT;
+    zq[u] = zigzag(quantize(X[tix<B>(q % B, (q / B) % B, q / (B * B))], step, inv, &bad));
+    zc[(size_t)c * B3 + q] = zq[u];
+    zsum += zq[u];
   }
+  if (bad) atomicOr(err, 1);
   const unsigned long long mean = block_sum_u64<NT>(zsum, red) / (unsigned long long)B3;
   int k = 0;
   while (k < 24 && (mean >> (k + 1)) != 0) ++k;
   unsigned long long bits = 0;
-  for (int q = threadIdx.x; q < B3; q += NT) bits += code_len(zc[(size_t)c * B3 + q], k);
+#pragma unroll
+  for (int u = 0; u < B3 / NT; ++u) bits += code_len(zq[u], k);
   const unsigned long long nbits = block_sum_u64<NT>(bits, red);
   if (threadIdx.x == 0) {
     cube_nbits[c] = (uint32_t)nbits;
@@ -432,11 +487,7 @@ __global__ __launch_bounds__(B * B) void k_wav_decode(const uint32_t* __restrict
   }
   if (t == 0 && valid < (uint32_t)B3) atomicOr(err, 2);
   __syncthreads();
-  for (int m = 2; m <= B; m *= 2)
-    for (int d = 2; d >= 0; --d) {
-      if (threadIdx.x < m * m) lift_inverse<B>(X, d, threadIdx.x % m, threadIdx.x / m, m);
-      __syncthreads();
-    }
+  wav_inverse<B, B>(X);
   for (int q = threadIdx.x; q < B3; q += NT)
     f[(size_t)c * B3 + q] = T(X[tix<B>(q % B, (q / B) % B, q / (B * B))]);
 }
@@ -460,8 +511,8 @@ cudaError_t compress_t(const Ctx& x, const void* field, double step, uint32_t* z
   auto kf = k_wav_forward<B, T>;
   cudaError_t e = wav_allow(kf, wav_smem<B>());
   if (e != cudaSuccess) return e;
-  kf<<<x.g.n_cubes, B * B, wav_smem<B>(), x.stream>>>((const T*)field, step, zc, cube_nbits,
-                                                      cube_k, err);
+  kf<<<x.g.n_cubes, B * B, wav_smem<B>(), x.stream>>>((const T*)field, step, wav_inv(step), zc,
+                                                      cube_nbits, cube_k, err);
   k_wav_offsets<<<1, 1024, 0, x.stream>>>(cube_nbits, nullptr, x.g.n_cubes, off);
   return cudaGetLastError();
 }
