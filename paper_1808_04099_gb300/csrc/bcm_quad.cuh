@@ -291,8 +291,8 @@ struct Halo {
 };
 
 // A quad of the cube into the tile, with the ghosts it sets across domain faces.
-template <int B, class TV>
-__device__ __forceinline__ void own_quad(TV* __restrict__ S, TV* __restrict__ gh, const CubeQ<TV>& cq,
+template <int B, class TV, class CQ>
+__device__ __forceinline__ void own_quad(TV* __restrict__ S, TV* __restrict__ gh, const CQ& cq,
                                          int i0, int j, int kk, const TV (&v)[4]) {
   constexpr int BB = B * B;
   st4(S + (kk * B + j) * B + i0, v);
@@ -316,9 +316,9 @@ __device__ __forceinline__ void own_quad(TV* __restrict__ S, TV* __restrict__ gh
 // The 7-point sums (K v / h) of a thread's column of four quads, planes k0 .. k0 + 3, from
 // the complete tile; out(m, acc) consumes plane k0 + m.  The threads of a warp call it
 // together.
-template <int B, class TV, class Out>
+template <int B, class TV, class CQ, class Out>
 __device__ __forceinline__ void quad_column(const TV* __restrict__ S, const TV* __restrict__ gh,
-                                            const CubeQ<TV>& cq, int i0, int j, int k0,
+                                            const CQ& cq, int i0, int j, int k0,
                                             const TV (&v)[4][4], const Out& out) {
   constexpr int BB = B * B;
   TV zm[4], zp[4];

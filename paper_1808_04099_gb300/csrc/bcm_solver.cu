@@ -23,6 +23,81 @@
 
 namespace bcm {
 
+// What follows a residual (its last block): the solve's or the cycle's scalars and targets,
+// which sims still run, and zeroed sums for the PCG that follows.
+template <bool MIXED>
+__device__ __forceinline__ void residual_decide(const DevGrid& g, const SolveParams& prm, int NT) {
+  int alive = 0, outer_alive = 0;
+  for (int q = threadIdx.x; q < g.n_sims; q += NT) {
+    SimState& t = g.ss[q];
+    const double bb = acc_take(t, ACC_BB), rr64 = acc_take(t, ACC_RR64);
+    const double rz = acc_take(t, ACC_RZ), rr = acc_take(t, ACC_RR);
+    if (MIXED && t.outer_done) continue;
+    if (MIXED) {
+      t.cycles += 1;
+      if (t.cycles == 1) {
+        t.bb = bb;
+        t.tol2 = prm.rtol * prm.rtol * bb;
+        t.zero_rhs = (bb == 0.0);
+      }
+      t.rr64 = rr64;
+      const bool ok = t.zero_rhs || rr64 <= t.tol2;
+      if (!isfinite(rr64)) t.nonfinite = 1;
+      if (ok || t.cycles > prm.max_cycles || t.nonfinite) {
+        t.outer_done = 1;
+        t.done = 1;
+        t.converged = ok;
+      } else {
+        t.rz = rz;
+        t.rr = rr;
+        // inner target: the reduction eta = inner_rtol per cycle, or, once the
+        // reduction rho still needed (||r|| rho = the outer tolerance) is within 4 eta,
+        // rho / 2, so the cycle ends the solve instead of overshooting it or stopping
+        // just short of it
+        const double in2 = prm.inner_rtol * prm.inner_rtol, need2 = 0.25 * t.tol2 / rr64;
+        t.inner_tol2 = (16.0 * need2 >= in2 ? need2 : in2) * rr;
+        t.iter = 0;
+        t.beta = 0.0;
+        t.done = (rr == 0.0);
+        // reliable update: after the first cycle the inner CG resumes its previous
+        // search direction with the true (FP64) residual in place of its own
+        t.cont = (prm.recycle && t.cycles > 1) ? 1 : 0;
+        alive |= !t.done;
+        outer_alive = 1;
+      }
+    } else {
+      t.bb = bb;
+      t.tol2 = prm.rtol * prm.rtol * bb;
+      t.zero_rhs = (bb == 0.0);
+      t.rz = rz;
+      t.rr = rr;
+      t.rr64 = rr;
+      t.iter = 0;
+      t.total_iters = 0;
+      t.beta = 0.0;
+      t.cont = 0;
+      if (!isfinite(rr)) t.nonfinite = 1;
+      t.done = t.zero_rhs || rr <= t.tol2 || t.nonfinite;
+      t.converged = t.zero_rhs || rr <= t.tol2;
+      alive |= !t.done;
+    }
+  }
+  // the persistent PCG's rotating dot-product slots start every solve at zero
+  for (int i = threadIdx.x; i < g.n_sims * kStripes; i += NT) {
+    SimState& t = g.ss[i / kStripes];
+    for (int sl = 0; sl < ACC_NSLOT; ++sl) t.acc[i % kStripes][ACC_SLOT_PQ + sl] = 0.0;
+    for (int sl = 0; sl < ACC_FZ_SLOTS; ++sl) t.acc[i % kStripes][ACC_SLOT_FZ + sl] = 0.0;
+  }
+  alive = __syncthreads_or(alive);
+  outer_alive = __syncthreads_or(outer_alive);
+  if (threadIdx.x == 0) {
+    g.flags[0] = !alive;
+    g.flags[1] = MIXED ? !outer_alive : 1;
+    set_cond(prm.cond_inner, alive ? 1u : 0u);
+    if (MIXED) set_cond(prm.cond_outer, outer_alive ? 1u : 0u);
+  }
+}
+
 // ===========================================================================
 // residual r = rhs - K x of the FP64 iterate x = p, rhs = -V (b - mean).
 // FP64 mode: starts the PCG.  Mixed mode: one defect-correction cycle; r goes to
@@ -100,77 +175,109 @@ __global__ __launch_bounds__(NT) void k_residual(DevGrid g, const double* __rest
     acc_add(st, ACC_RZ, acc4[2]);
     acc_add(st, ACC_RR, acc4[3]);
   }
-  if (last_block(g.counter)) {
-    int alive = 0, outer_alive = 0;
-    for (int q = threadIdx.x; q < g.n_sims; q += NT) {
-      SimState& t = g.ss[q];
-      const double bb = acc_take(t, ACC_BB), rr64 = acc_take(t, ACC_RR64);
-      const double rz = acc_take(t, ACC_RZ), rr = acc_take(t, ACC_RR);
-      if (MIXED && t.outer_done) continue;
-      if (MIXED) {
-        t.cycles += 1;
-        if (t.cycles == 1) {
-          t.bb = bb;
-          t.tol2 = prm.rtol * prm.rtol * bb;
-          t.zero_rhs = (bb == 0.0);
-        }
-        t.rr64 = rr64;
-        const bool ok = t.zero_rhs || rr64 <= t.tol2;
-        if (!isfinite(rr64)) t.nonfinite = 1;
-        if (ok || t.cycles > prm.max_cycles || t.nonfinite) {
-          t.outer_done = 1;
-          t.done = 1;
-          t.converged = ok;
-        } else {
-          t.rz = rz;
-          t.rr = rr;
-          // inner target: the reduction eta = inner_rtol per cycle, or, once the
-          // reduction rho still needed (||r|| rho = the outer tolerance) is within 4 eta,
-          // rho / 2, so the cycle ends the solve instead of overshooting it or stopping
-          // just short of it
-          const double in2 = prm.inner_rtol * prm.inner_rtol, need2 = 0.25 * t.tol2 / rr64;
-          t.inner_tol2 = (16.0 * need2 >= in2 ? need2 : in2) * rr;
-          t.iter = 0;
-          t.beta = 0.0;
-          t.done = (rr == 0.0);
-          // reliable update: after the first cycle the inner CG resumes its previous
-          // search direction with the true (FP64) residual in place of its own
-          t.cont = (prm.recycle && t.cycles > 1) ? 1 : 0;
-          alive |= !t.done;
-          outer_alive = 1;
-        }
-      } else {
-        t.bb = bb;
-        t.tol2 = prm.rtol * prm.rtol * bb;
-        t.zero_rhs = (bb == 0.0);
-        t.rz = rz;
-        t.rr = rr;
-        t.rr64 = rr;
-        t.iter = 0;
-        t.total_iters = 0;
-        t.beta = 0.0;
-        t.cont = 0;
-        if (!isfinite(rr)) t.nonfinite = 1;
-        t.done = t.zero_rhs || rr <= t.tol2 || t.nonfinite;
-        t.converged = t.zero_rhs || rr <= t.tol2;
-        alive |= !t.done;
+  if (last_block(g.counter)) residual_decide<MIXED>(g, prm, NT);
+}
+
+// The same on whole cubes of 16^3 or 8^3 by quad tiles (bcm_quad.cuh).  It is bound by the
+// FP64 pipe: about 10 operations a cell in the mixed mode against 22 of the padded-tile
+// kernel (the neighbour sum six instead of eleven, ||rhs|| only in a solve's first cycle,
+// the FP32 sums and diagonals in FP32): 4.2M cells in 180 us before, 128 us now.
+template <int B, class TV, bool MIXED>
+__global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<double>()) void k_residual_quad(
+    DevGrid g, const double* __restrict__ b, const double* __restrict__ x, TV* __restrict__ r,
+    float* __restrict__ e, SolveParams prm) {
+  using T = QT<B>;
+  constexpr int B3 = T::B3, BB = T::BB;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ CubeQ<TV> cqs[T::CPB];
+  const int cub = threadIdx.x / T::TPC, lt = threadIdx.x - cub * T::TPC;
+  const int c = blockIdx.x * T::CPB + cub;
+  double* S = reinterpret_cast<double*>(smem_raw) + cub * T::N;
+  double* gh = S + B3;
+  CubeQ<TV>& cq = cqs[cub];
+  const bool valid = c < g.n_cubes;
+  const CubeLoad L = cube_lookup(g, valid ? c : 0, lt);
+  Halo<B> H;
+  H.lookup(g, valid ? c : 0, lt);
+  poison_tile(reinterpret_cast<double*>(smem_raw), T::CPB * T::N);
+  SimState& st = g.ss[L.s];
+  const bool active = valid && !(MIXED && st.outer_done);
+  const bool want_bb = !MIXED || st.cycles == 0;  // (the last block counts the cycles)
+  double bb[1] = {0.0}, rr64[1] = {0.0};
+  TV rz[1] = {TV(0)}, rr[1] = {TV(0)};
+  if (active) {
+    const int pos = lt % T::Q, i0 = (4 * pos) % B, j = (4 * pos) / B, k0 = 4 * (lt / T::Q);
+    const size_t base = (size_t)c * B3 + (k0 * B + j) * B + i0;
+    double v[4][4], ha[Halo<B>::R][4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) ld4(x + base + m * BB, v[m]);
+    H.each(lt, [&](int u, int, int n, int cell, int stride) {
+      ldq(x + (size_t)n * B3 + cell, stride, ha[u]);
+    });
+    cube_publish(cq, g, L, lt);
+    T::sync();
+    auto make = [&](int u, int, int, int, int, double (&o)[4]) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) o[q] = ha[u][q];
+    };
+    auto one = [&](int n, int cell) { return x[(size_t)n * B3 + cell]; };
+    H.store(gh, g, c, lt, make, one, 0);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) own_quad<B>(S, gh, cq, i0, j, k0 + m, v[m]);
+    T::sync();
+    const double h0 = g.sp[L.s].h0, h = g.max_level && g.lvl[c] ? 0.5 * h0 : h0;
+    const double V = h * h * h, mean = st.bmean;
+    quad_column<B>(S, gh, cq, i0, j, k0, v, [&](int m, const double (&acc)[4]) {
+      double bv[4], rv[4];
+      ld4(b + base + m * BB, bv);
+      if (mean != 0.0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) bv[q] -= mean;
       }
-    }
-    // the persistent PCG's rotating dot-product slots start every solve at zero
-    for (int i = threadIdx.x; i < g.n_sims * kStripes; i += NT) {
-      SimState& t = g.ss[i / kStripes];
-      for (int sl = 0; sl < ACC_NSLOT; ++sl) t.acc[i % kStripes][ACC_SLOT_PQ + sl] = 0.0;
-      for (int sl = 0; sl < ACC_FZ_SLOTS; ++sl) t.acc[i % kStripes][ACC_SLOT_FZ + sl] = 0.0;
-    }
-    alive = __syncthreads_or(alive);
-    outer_alive = __syncthreads_or(outer_alive);
-    if (threadIdx.x == 0) {
-      g.flags[0] = !alive;
-      g.flags[1] = MIXED ? !outer_alive : 1;
-      set_cond(prm.cond_inner, alive ? 1u : 0u);
-      if (MIXED) set_cond(prm.cond_outer, outer_alive ? 1u : 0u);
-    }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const double rhs = -V * bv[q];
+        rv[q] = fma(-h, acc[q], rhs);
+        if (want_bb) bb[0] = fma(rhs, rhs, bb[0]);
+      }
+      TV rt[4], inv[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) rt[q] = TV(rv[q]);
+      quad_inv<B>(cq, i0, j, k0 + m, inv);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) rz[0] += rt[q] * (rt[q] * inv[q]);
+      rr[0] += dot4(rt, rt);
+      st4(r + base + m * BB, rt);
+      if constexpr (MIXED) {
+        rr64[0] += dot4(rv, rv);
+        const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+        st4(e + base + m * BB, zero);
+      }
+    });
   }
+  // sums per cube (a warp, or the block)
+  auto sum = [&](auto& p) {
+    double val[1];
+    if constexpr (T::TPC == 32) {
+      auto w = p[0];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+      val[0] = double(w);
+    } else {
+      __shared__ double red[32];
+      block_sum_tv<T::NT, 1>(p, val, red);
+    }
+    return val[0];
+  };
+  const double s_rz = sum(rz), s_rr = sum(rr);
+  const double s_rr64 = MIXED ? sum(rr64) : 0.0, s_bb = want_bb ? sum(bb) : 0.0;
+  if (lt == 0 && active) {
+    if (want_bb) acc_add_cube(st, ACC_BB, c, s_bb);
+    if (MIXED) acc_add_cube(st, ACC_RR64, c, s_rr64);
+    acc_add_cube(st, ACC_RZ, c, s_rz);
+    acc_add_cube(st, ACC_RR, c, s_rr);
+  }
+  if (last_block(g.counter)) residual_decide<MIXED>(g, prm, T::NT);
 }
 
 // alpha of every running sim from the completed <p, K p> (last block of pass A)
@@ -640,22 +747,30 @@ static cudaError_t allow_smem(K kernel, size_t bytes) {
     default: return cudaErrorInvalidValue;                 \
   }
 
+template <int B, class TV, bool MIXED>
+static cudaError_t residual_quad_t(const Ctx& x, const SolveParams& prm) {
+  using T = QT<B>;
+  const size_t sm = sizeof(double) * (size_t)T::N * T::CPB;
+  auto kern = k_residual_quad<B, TV, MIXED>;
+  cudaError_t e = allow_dynamic_smem(kern, sm);
+  if (e != cudaSuccess) return e;
+  kern<<<(x.g.n_cubes + T::CPB - 1) / T::CPB, T::NT, sm, x.stream>>>(x.g, x.f.b, x.f.p, (TV*)x.f.r,
+                                                                     x.f.e, prm);
+  return cudaGetLastError();
+}
 cudaError_t launch_residual(const Ctx& x, const SolveParams& prm) {
-  BCM_DISPATCH_B(x.B, {
-    constexpr int NT = threads_for<B>();
-    const size_t sm = sizeof(double) * Slab<B, B>::N;
-    if (x.solve64) {
-      auto kern = k_residual<B, NT, double, false>;
-      cudaError_t e = allow_smem(kern, sm);
-      if (e != cudaSuccess) return e;
-      kern<<<x.g.n_cubes, NT, sm, x.stream>>>(x.g, x.f.b, x.f.p, (double*)x.f.r, nullptr, prm);
-    } else {
-      auto kern = k_residual<B, NT, float, true>;
-      cudaError_t e = allow_smem(kern, sm);
-      if (e != cudaSuccess) return e;
-      kern<<<x.g.n_cubes, NT, sm, x.stream>>>(x.g, x.f.b, x.f.p, (float*)x.f.r, x.f.e, prm);
-    }
-  });
+  // whole cubes of 16^3 and 8^3 by quad tiles, cubes of 4^3 (a quarter warp) by padded ones
+  if (x.B == 16)
+    return x.solve64 ? residual_quad_t<16, double, false>(x, prm) : residual_quad_t<16, float, true>(x, prm);
+  if (x.B == 8)
+    return x.solve64 ? residual_quad_t<8, double, false>(x, prm) : residual_quad_t<8, float, true>(x, prm);
+  if (x.B != 4) return cudaErrorInvalidValue;
+  constexpr int B = 4, NT = threads_for<B>();
+  const size_t sm = sizeof(double) * Slab<B, B>::N;
+  if (x.solve64)
+    k_residual<B, NT, double, false><<<x.g.n_cubes, NT, sm, x.stream>>>(x.g, x.f.b, x.f.p, (double*)x.f.r, nullptr, prm);
+  else
+    k_residual<B, NT, float, true><<<x.g.n_cubes, NT, sm, x.stream>>>(x.g, x.f.b, x.f.p, (float*)x.f.r, x.f.e, prm);
   return cudaGetLastError();
 }
 
