@@ -29,7 +29,12 @@
 
 namespace bcm {
 
-constexpr int kCubeCache = 4;  // cubes whose constants a block keeps for the whole solve
+// Cubes whose constants a block keeps for the whole solve; a block with more of them loads a
+// cube's constants again for every item of both passes (two round trips and a barrier).
+// Microseconds per iteration with 4, 8 and 40: 8.4M cells (4 cubes on the fullest block) 63,
+// 64, 65; 10.4M on two levels (5) 120, 104, 109; 16.8M (7) 139, 124, 126 (40 take their
+// shared memory from the L1 cache).
+constexpr int kCubeCache = 8;
 
 template <int B, int KS, int NT, class TV, class TX>
 __global__ __launch_bounds__(NT, 4) void k_pcg(DevGrid g, TX* __restrict__ x, TV* __restrict__ r,
