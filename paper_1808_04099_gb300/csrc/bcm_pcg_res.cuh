@@ -921,6 +921,9 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
         st4(x + base + c0, xv);
       }
     }
+    // Several sims: the warps of the next decisions set ResSim::done, which the loop above
+    // reads, as soon as their sim's words are there (with one sim a barrier comes first).
+    if (multi) __syncthreads();
   }
   if (failed) return;
   // ---- exit: the iterate (mixed: added to the FP64 one), and in mixed mode the search
