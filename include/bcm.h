@@ -245,6 +245,15 @@ bcm_status bcm_get_solver(const bcm_grid *grid, double *inner_rtol, int32_t *max
  * BCM_E_INVALID for other values. */
 bcm_status bcm_set_launch(bcm_grid *grid, int persistent, int slabs_a, int slabs_b);
 
+/* Test path, no GPU needed: the launch shape of the on-chip PCG (FP64 vectors, or those of
+ * the FP32 inner solve) for a grid of these sizes on a device of n_sms SMs whose blocks may
+ * use smem_bytes of dynamic shared memory.  Returns 0 when the grid does not fit, else 1
+ * and out[6]: planes of a work item (a z-slab of a cube), blocks, items of the fullest
+ * block, threads per block, quads of cells per thread, the cube edge whose unrolled kernel
+ * runs (0: the general one). */
+int bcm_onchip_shape(int cells_per_edge, int n_cubes, int n_sims, int max_level, int fp64,
+                     int n_sms, size_t smem_bytes, int32_t *out);
+
 /* z-slabs per 16^3 cube of the momentum and Poisson right-hand-side kernels (one block
  * per slab, its tiles of u*, v*, w* with their halos in shared memory): 1, 2 or 4; 0
  * the default (2 in FP32, 4 in FP64).  Other cube sizes take whole cubes (the value is

@@ -24,7 +24,7 @@ SCHEME_AB2_CENTRAL, SCHEME_QUICK_CN = 0, 1
 
 EXPORTED = ["bcm_workspace_bytes", "bcm_create_grid", "bcm_destroy_grid", "bcm_field",
             "bcm_set_geometry", "bcm_reset_time", "bcm_drag_mean", "bcm_set_solver",
-            "bcm_set_launch", "bcm_set_stencil_slabs", "bcm_get_stencil_slabs",
+            "bcm_set_launch", "bcm_onchip_shape", "bcm_set_stencil_slabs", "bcm_get_stencil_slabs",
             "bcm_set_preconditioner", "bcm_apply_preconditioner",
             "bcm_set_step", "bcm_get_solver", "bcm_measure_fma_rate", "bcm_step", "bcm_step_graph", "bcm_solve_pressure",
             "bcm_adjoint_bytes", "bcm_adjoint_init", "bcm_adjoint_step",
@@ -108,6 +108,7 @@ def lib(build: bool = True):
                                        C.c_int, P]
         L.bcm_set_solver.argtypes = [P, C.c_double, C.c_int, C.c_int, C.c_double, C.c_int]
         L.bcm_set_launch.argtypes = [P, C.c_int, C.c_int, C.c_int]
+        L.bcm_onchip_shape.argtypes = [C.c_int] * 6 + [C.c_size_t, P]
         L.bcm_set_stencil_slabs.argtypes = [P, C.c_int]
         L.bcm_get_stencil_slabs.argtypes = [P, P]
         L.bcm_get_solver.argtypes = [P, P, P, P, P, P]
@@ -158,6 +159,16 @@ def _body_struct(b) -> Body:
     s.omega[:] = list(map(float, b.omega))
     s.vel[:] = list(map(float, b.vel))
     return s
+
+
+def onchip_shape(B: int, n_cubes: int, n_sims: int = 1, max_level: int = 0, fp64: bool = True,
+                 n_sms: int = 152, smem: int = 229824) -> Optional[dict]:
+    """Launch shape of the on-chip PCG for a grid of these sizes, None when it does not fit
+    (no GPU needed; the defaults are those of GB300)."""
+    v = (C.c_int32 * 6)()
+    if not lib().bcm_onchip_shape(B, n_cubes, n_sims, max_level, int(fp64), n_sms, smem, v):
+        return None
+    return dict(zip(("planes", "blocks", "items", "threads", "quads", "edge"), v))
 
 
 def fma_rate(fp64: bool = True) -> float:

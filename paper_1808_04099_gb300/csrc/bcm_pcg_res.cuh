@@ -512,7 +512,7 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
 
   // Sums of NV values per thread (several sims: per thread and quad), published under
   // exchange number n.  One sim: t[] is the thread's sum.  Several: each quad's values
-  // were reduced over units of 16 quads, which never cross an item, into red[].
+  // were reduced over units of 16 quads, which never cross an item (res_shape), into red[].
   auto unit_sum = [&](int unit, int a, TV t) {
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
@@ -983,6 +983,8 @@ bool res_shape(const Ctx& x, int nsm, size_t smem_max, ResPlan* out) {
     const int KS = 1 << lk, IC = B * B * KS, G = 4 * KS * B + 2 * B * B;
     const long long N = (long long)x.g.n_cubes * (B / KS);
     if (N * G > 0x7fffffffLL) continue;
+    // with several sims the sums run over units of 64 cells, which must not cross items
+    if (x.g.n_sims > 1 && IC < 64) continue;
     for (int div = 1; div <= 16; ++div) {
       const int most = (blocks + div - 1) / div;
       const int grid = N < most ? (int)N : most;

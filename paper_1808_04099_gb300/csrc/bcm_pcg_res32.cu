@@ -31,3 +31,23 @@ cudaError_t launch_pcg_resident(const Ctx& x, const SolveParams& prm, bool* laun
 }
 
 }  // namespace bcm
+
+extern "C" int bcm_onchip_shape(int cells_per_edge, int n_cubes, int n_sims, int max_level, int fp64,
+                                int n_sms, size_t smem_bytes, int32_t* out) {
+  using namespace bcm;
+  if (!out || n_cubes < 1 || n_sims < 1 || n_sims > n_cubes || n_sms < 1 ||
+      (cells_per_edge != 4 && cells_per_edge != 8 && cells_per_edge != 16))
+    return 0;
+  Ctx x{};
+  x.B = cells_per_edge;
+  x.g.n_cubes = n_cubes;
+  x.g.n_sims = n_sims;
+  x.g.max_level = max_level;
+  ResPlan P{};
+  if (n_sims > kMaxPersistentSims || !(fp64 ? res_shape<double>(x, n_sms, smem_bytes, &P)
+                                            : res_shape<float>(x, n_sms, smem_bytes, &P)))
+    return 0;
+  const int32_t v[6] = {1 << P.sh.lk, P.grid, P.sh.ipb, P.nt, P.m, P.geo};
+  for (int i = 0; i < 6; ++i) out[i] = v[i];
+  return 1;
+}

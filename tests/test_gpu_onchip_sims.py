@@ -1,11 +1,14 @@
 """On-chip PCG with several sims per block: sims of one block that converge at different
 iterations each return the iterate that their reported residual belongs to (the last
 x += alpha p of a sim is not lost to the decisions of the next iteration), with x in
-registers and in global memory, whatever the number of sims of a block."""
+registers and in global memory, whatever the number of sims of a block; and two sims of
+4^3 cubes, in numbers of cubes for which half cubes would spread the cells better, give the
+two-launch form's iterates (every cell is in its sim's dot products)."""
 import numpy as np
 import pytest
 
 from paper_1808_04099_gb300 import workloads as W
+from _util import rel_l2
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -69,3 +72,28 @@ def test_reported_residual_is_that_of_the_iterate(name):
         # by rounding, under 2^-53 * 12 |p| h / |rhs| <= 12 * 2^-53 N^2 / pi^2 for N <= 48
         # cells along a sim: 4e-13.  Without its last update an iterate stands above RTOL.
         assert rel.max() <= RTOL * 1.01, (seed, int(rel.argmax()), rel.max())
+
+
+@pytest.mark.parametrize("prec,tol", [(bcm.PREC_F64, 1e-12), (bcm.PREC_F32_REFINE, 1e-5)])
+@pytest.mark.parametrize("sizes", [((1, 1, 1), (1, 1, 1)), ((2, 2, 2), (3, 2, 1)),
+                                   ((2, 2, 2), (7, 1, 1)), ((7, 2, 2), (7, 2, 2)),
+                                   ((5, 4, 3), (5, 4, 3)), ((10, 5, 5), (10, 5, 5))])
+def test_two_sims_of_small_cubes(sizes, prec, tol):
+    spec = W.concat([channel(*n, 4) for n in sizes])
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(7)
+    rhs = torch.randn(spec.n_cells, generator=gen, device="cuda", dtype=torch.float64)
+
+    def iterate(k, form):
+        g = bcm.Grid(spec, prec)
+        if form == 0:
+            g.set_launch(1, 1, persistent=0)
+        g.set_solver(inner_rtol=1e-30, max_cycles=1)
+        g.field(bcm.RHS).copy_(rhs)
+        g.field(bcm.P).zero_()
+        st = g.solve_pressure_iters(k)
+        assert all(s["pcg_form"] == form and s["cg_iters"] == k for s in st)
+        return g.numpy(bcm.P)
+
+    for k in (1, 4):
+        assert rel_l2(iterate(k, 3), iterate(k, 0)) <= tol, k
