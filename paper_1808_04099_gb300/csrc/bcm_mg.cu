@@ -1049,12 +1049,20 @@ static cudaError_t up_quad_t(const Ctx& x, int l, const SolveParams& prm, int mo
                     l == 0 ? 1 : 0, l);
 }
 
-// First level of the coarse kernel: at most 4^3 cells per cube, and no more cells than the
-// largest cluster has threads (a launch over all SMs does more of them faster).
+// First level of the coarse kernel: at most 4^3 cells per cube, and at most kCoarseCells cells
+// (a launch over all SMs does more of them faster).  A block takes kCoarseBlock cells, up to
+// the largest cluster: one SM does 1.7 FP64 operations a clock, so with 1024 cells a block
+// these levels took longer than the launches they replaced.  FP64 steps in us with a launch
+// per level, with 16k cells and 1024 a block, and with these: 128 cubes of 4^3 2031, 2312,
+// 1868; 1728 of 4^3 3408, 3485, 3128; 16 of 8^3 2577, 2998, 2556; 128 of 8^3 3341, 3592,
+// 3084; 1024 of 16^3 31.4, 24.9, 24.3 ms.  2048 and 1024 cells, 256 and 64 a block: the same
+// within 2 %.
+constexpr long long kCoarseCells = 4096;
+constexpr long long kCoarseBlock = 128;
 static int coarse_from(const Ctx& x) {
   int l = 1;
   while (l < x.mg.L && ((x.B >> l) > 4 || (long long)x.g.n_cubes * (x.B >> l) * (x.B >> l) * (x.B >> l) >
-                                              16LL * 1024))
+                                              kCoarseCells))
     ++l;
   return l;
 }
@@ -1065,8 +1073,8 @@ static cudaError_t coarse_t(const Ctx& x, int lf, int all) {
   while (kd < x.mg.M && (x.mg.n[kd] > 1024 || agg_smem(x.mg, x.g.n_cubes, kd) > 200 * 1024)) ++kd;
   const size_t sm = agg_smem(x.mg, x.g.n_cubes, kd);
   const long long bl = x.B >> lf, cells = x.g.n_cubes * bl * bl * bl;
-  int ranks = 1;  // a cell per thread, up to the largest cluster
-  while (ranks < 16 && (cells > 1024LL * ranks || (kd > 0 && x.mg.n[0] > 1024 * ranks))) ranks *= 2;
+  int ranks = 1;
+  while (ranks < 16 && (cells > kCoarseBlock * ranks || (kd > 0 && x.mg.n[0] > 1024 * ranks))) ranks *= 2;
   auto kern = k_mg_coarse<TV>;
   cudaError_t e = allow_dynamic_smem(kern, sm);
   if (e != cudaSuccess) return e;
