@@ -812,6 +812,7 @@ extern "C" bcm_status bcm_create_grid(const bcm_grid_desc* desc, void* dev_works
       D.cidx[k] = (int*)(W + ml.cidx[k]);
       D.parent[k] = (int*)(W + ml.parent[k]);
     }
+    D.cluster_max = mg_cluster_limit(x);
   }
   *out = g;
   return BCM_OK;

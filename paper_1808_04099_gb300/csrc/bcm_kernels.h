@@ -77,6 +77,7 @@ constexpr int kMgNuTop = 4;       // Jacobi sweeps on the top aggregate level
 constexpr double kMgOver = 1.75;  // scale of the coarse-grid correction
 struct MgDev {
   int L, M;
+  int cluster_max;       // blocks of the coarse kernel's largest cluster (mg_cluster_limit)
   void* x[kMgMaxL + 1];  // pre-smoothed iterate of level l
   void* y[kMgMaxL + 1];  // corrected iterate of level l (y[0] = z, the PCG's M^-1 r)
   void* r[kMgMaxL + 1];  // residual of level l (r[0] is the PCG residual)
@@ -171,6 +172,7 @@ cudaError_t launch_apply_poisson(const Ctx& x, const double* in, double* out);
 // (<r,z> becomes the PCG's rz); 1: after pass A, doing pass B too (<r,r>), then <r,z>,
 // beta and the convergence decision; 2: standalone (every sim, no dot products).
 cudaError_t launch_mg_vcycle(const Ctx& x, const SolveParams& prm, int mode);
+int mg_cluster_limit(const Ctx& x);  // (sizes and the device's answer only: at grid creation)
 // Lagrangian particles: per-cube sets from the positions (counting sort); the
 // forcing sub-step (interpolation of u~, F, spreading into u*); the position update.
 cudaError_t launch_ib_bin(const Ctx& x);

@@ -1066,34 +1066,68 @@ static int coarse_from(const Ctx& x) {
     ++l;
   return l;
 }
-template <class TV>
-static cudaError_t coarse_t(const Ctx& x, int lf, int all) {
-  // aggregate levels of more than 1024 nodes, or that do not fit, run on the cluster
+// aggregate levels of more than 1024 nodes, or that do not fit a block's shared memory, run on
+// the cluster: levels k < coarse_kd
+static int coarse_kd(const Ctx& x) {
   int kd = 0;
   while (kd < x.mg.M && (x.mg.n[kd] > 1024 || agg_smem(x.mg, x.g.n_cubes, kd) > 200 * 1024)) ++kd;
-  const size_t sm = agg_smem(x.mg, x.g.n_cubes, kd);
-  const long long bl = x.B >> lf, cells = x.g.n_cubes * bl * bl * bl;
-  int ranks = 1;
-  while (ranks < 16 && (cells > kCoarseBlock * ranks || (kd > 0 && x.mg.n[0] > 1024 * ranks))) ranks *= 2;
+  return kd;
+}
+// The coarse kernel's launch as one cluster of `ranks` blocks; at: two attributes for cfg.
+template <class TV>
+static cudaError_t coarse_config(const Ctx& x, int ranks, cudaLaunchAttribute* at,
+                                 cudaLaunchConfig_t* cfg) {
+  const size_t sm = agg_smem(x.mg, x.g.n_cubes, coarse_kd(x));
   auto kern = k_mg_coarse<TV>;
   cudaError_t e = allow_dynamic_smem(kern, sm);
   if (e != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
     return e;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(ranks);
-  cfg.blockDim = dim3(1024);
-  cfg.dynamicSmemBytes = sm;
-  cfg.stream = x.stream;
-  cudaLaunchAttribute at[2];
+  cfg->gridDim = dim3(ranks);
+  cfg->blockDim = dim3(1024);
+  cfg->dynamicSmemBytes = sm;
+  cfg->stream = x.stream;
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = ranks;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kern, x.g, x.mg, lf, (int)bl, kd, all);
+  cfg->attrs = at;
+  cfg->numAttrs = 2;
+  return cudaSuccess;
+}
+template <class TV>
+static int coarse_limit_t(const Ctx& x) {
+  for (int ranks = 16; ranks > 1; ranks /= 2) {
+    cudaLaunchAttribute at[2];
+    cudaLaunchConfig_t cfg{};
+    int n = 0;
+    cudaError_t e = coarse_config<TV>(x, ranks, at, &cfg);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_mg_coarse<TV>, &cfg);
+    if (e == cudaSuccess && n >= 1) return ranks;
+    (void)cudaGetLastError();
+  }
+  return 1;
+}
+// Blocks of the largest cluster of the coarse kernel that the device runs for this grid: a
+// device or partition may have fewer than 16 SMs in one GPC with the shared memory free (one
+// block does all of it too).
+int mg_cluster_limit(const Ctx& x) {
+  return x.solve64 ? coarse_limit_t<double>(x) : coarse_limit_t<float>(x);
+}
+template <class TV>
+static cudaError_t coarse_t(const Ctx& x, int lf, int all) {
+  const int kd = coarse_kd(x);
+  const long long bl = x.B >> lf, cells = x.g.n_cubes * bl * bl * bl;
+  int ranks = 1;
+  while (ranks < x.mg.cluster_max &&
+         (cells > kCoarseBlock * ranks || (kd > 0 && x.mg.n[0] > 1024 * ranks)))
+    ranks *= 2;
+  cudaLaunchAttribute at[2];
+  cudaLaunchConfig_t cfg{};
+  const cudaError_t e = coarse_config<TV>(x, ranks, at, &cfg);
+  if (e != cudaSuccess) return e;
+  return cudaLaunchKernelEx(&cfg, k_mg_coarse<TV>, x.g, x.mg, lf, (int)bl, kd, all);
 }
 
 template <class TV>
