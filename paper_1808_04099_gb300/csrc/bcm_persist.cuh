@@ -108,14 +108,21 @@ __device__ __forceinline__ void warp_slot_sums(SimState& st, int idx_a, int idx_
 
 // Dynamic shared memory beyond the default limit (48 KB minus the kernel's static
 // shared memory) needs the kernel's opt-in.
+// The opt-in is per kernel and not per launch, so it is always raised to all that the device
+// gives: one thread's smaller grid does not lower it between another's opt-in and launch.
 template <class K>
 inline cudaError_t allow_dynamic_smem(K kern, size_t dyn) {
   cudaFuncAttributes fa;
   cudaError_t e = cudaFuncGetAttributes(&fa, kern);
   if (e != cudaSuccess) return e;
-  if (fa.sharedSizeBytes + dyn > 48 * 1024)
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-  return cudaSuccess;
+  if (fa.sharedSizeBytes + dyn <= 48 * 1024) return cudaSuccess;
+  int dev = 0, most = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
+    return e;
+  if (fa.sharedSizeBytes + dyn > (size_t)most) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              most - (int)fa.sharedSizeBytes);
 }
 
 // Launch with programmatic dependent launch: the kernel may be scheduled while the
