@@ -109,7 +109,7 @@ struct ResItem {
 
 struct ResSim {
   double alpha, beta, rz, rrz;  // rrz = 1 / rz
-  double rz0, rr0, tol2;        // <r, z>, <r, r> at entry, the target
+  double rz0, rr, tol2;         // <r, z> at entry, <r, r> of the last decision, the target
   int kdone;           // iterations this launch ran
   int done, first;
   int e0, cnt;         // the sim's words: first index and number of blocks
@@ -371,7 +371,7 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
     S.alpha = S.beta = 0.0;
     S.rz = cont ? st.rz_last : st.rz;
     S.rz0 = st.rz;
-    S.rr0 = st.rr;
+    S.rr = st.rr;
     S.tol2 = inner ? st.inner_tol2 : st.tol2;
     S.rrz = S.rz != 0.0 ? 1.0 / S.rz : 0.0;
     S.done = st.done ? 1 : 0;
@@ -576,35 +576,39 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
   using One = std::integral_constant<int, 1>;
   using Two = std::integral_constant<int, 2>;
 
-  // decisions of sim l from the sums of the previous pass B (lane 0 of a warp; the same
-  // in every block)
+  // the end of sim l after k iterations (lane 0 of a warp; the same in every block)
+  auto finish = [&](int l, int k, double rr, bool ok, bool bad) {
+    ResSim& S = sims[l];
+    SimState& st = g.ss[sim_lo + l];
+    S.done = 1;
+    S.kdone = k;
+    if (bl + sim_lo + l != S.e0) return;  // the sim's first block writes the results
+    st.iter = k;
+    st.total_iters += k;
+    st.rr = rr;
+    st.done = 1;
+    st.rz_last = S.rz;
+    st.p_off = 0;
+    if (bad) st.nonfinite = 1;
+    if (!inner) {
+      st.rr64 = rr;
+      st.converged = ok;
+    }
+  };
+  // decisions of sim l from the sums of the previous pass B
   auto decide = [&](int l, int k, double rz, double rr) {
     ResSim& S = sims[l];
     if (k == 0) {
       rz = S.rz0;
-      rr = S.rr0;
+      rr = S.rr;
     }
     const double tol2 = S.tol2;
     const bool bad = !isfinite(rr) || !isfinite(rz);
     if (bad || rr <= tol2 || k >= kmax) {
-      SimState& st = g.ss[sim_lo + l];
-      S.done = 1;
-      S.kdone = k;
-      if (bl + sim_lo + l == S.e0) {  // the sim's first block writes the results
-        st.iter = k;
-        st.total_iters += k;
-        st.rr = rr;
-        st.done = 1;
-        st.rz_last = S.rz;
-        st.p_off = 0;
-        if (bad) st.nonfinite = 1;
-        if (!inner) {
-          st.rr64 = rr;
-          st.converged = !bad && rr <= tol2;
-        }
-      }
+      finish(l, k, rr, !bad && rr <= tol2, bad);
       return;
     }
+    S.rr = rr;
     S.beta = ((k == 0 && S.first) || S.rz == 0.0) ? 0.0 : quick_div<TV>(rz, S.rz, S.rrz);
     S.rz = rz;
   };
@@ -819,12 +823,18 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
     }
     // (no fence: nothing another block reads has been written since the last exchange)
     publish(One{}, wa, nb, false, pq);
-    auto set_alpha = [&](ResSim& S, double (&va)[1][kWaitPer]) {
+    // A non-finite <p, Kp> ends an FP64 solve before it touches x, as in the two-launch form
+    // (the FP32 inner solve runs on with alpha = 0, as the streaming form does).
+    auto set_alpha = [&](int l, double (&va)[1][kWaitPer]) {
+      ResSim& S = sims[l];
       double s[1];
       words_sum<1>(va, S.cnt, s);
       // lane 0: alpha = <r, z> / <p, Kp>; lane 1: 1 / <r, z> for the next beta
       const double d = lane == 0 ? s[0] : S.rz, y = quick_rcp<TV>(d);
-      if (lane == 0) S.alpha = (d != 0.0 && isfinite(d)) ? quick_div<TV>(S.rz, d, y) : 0.0;
+      if (lane == 0) {
+        S.alpha = (d != 0.0 && isfinite(d)) ? quick_div<TV>(S.rz, d, y) : 0.0;
+        if (kD && !isfinite(d)) finish(l, k, S.rr, false, true);
+      }
       if (lane == 1) S.rrz = y;
     };
     double va[1][kWaitPer];
@@ -835,7 +845,7 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
       __syncthreads();
       if (warp == 0) {
         wval_load<1>(wval, sims[0].cnt, va);
-        set_alpha(sims[0], va);
+        set_alpha(0, va);
       }
     } else {
       for (int l = warp; l < nls; l += NW) {
@@ -845,7 +855,7 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
           if (lane == 0) s_fail = 1;
           continue;
         }
-        set_alpha(sims[l], va);
+        set_alpha(l, va);
       }
     }
     __syncthreads();
@@ -853,6 +863,7 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
       failed = true;
       break;
     }
+    if (kD && !multi && sims[0].done) break;
     // ---- pass B: z -= alpha M^-1 K p, face planes, <r, z>, <r, r>
     TV rs[2] = {TV(0), TV(0)};
     const int tid_b = opaque();
