@@ -1092,13 +1092,13 @@ bcm_status solve(bcm_grid* g, double rtol, int max_iter) {
     return BCM_OK;
   }
   if (g->solve64 && !mg && x.auto_form) {  // FP64 on chip where it fits, else two launches
-    bool launched = false;
-    RUN(BCM_K_PCG, launch_pcg_resident(x, prm, &launched));
-    if (launched) {
+    bool on_chip = false;
+    CUDA_TRY(pcg_resident_fits(x, &on_chip));
+    if (on_chip) {
+      RUN(BCM_K_PCG, launch_pcg_resident(x, prm, &on_chip));
       g->pcg_form = PCG_RESIDENT;
       return read_err(g);
     }
-    g->launch_count -= 1;
   }
   if ((st = read_flags(g, flags)) != BCM_OK) return st;
   if (g->solve64) {

@@ -158,6 +158,7 @@ cudaError_t launch_pcg1(const Ctx& x, const SolveParams& prm);
 // its correction to the FP64 iterate (SolveParams::x64_add), like the streaming form.
 cudaError_t launch_pcg_resident(const Ctx& x, const SolveParams& prm, bool* launched);
 cudaError_t launch_pcg_resident64(const Ctx& x, const SolveParams& prm, bool* launched);
+cudaError_t pcg_resident_fits(const Ctx& x, bool* fits);  // whether it would launch
 size_t res_words_bytes(int n_sims);
 inline bool adds_correction(int form) { return form == PCG_STREAMING || form == PCG_RESIDENT; }
 // The fused single-barrier form (FP32 inner solve, 16^3 cubes); *launched = false when

@@ -22,6 +22,13 @@ static cudaError_t res32(const Ctx& x, const SolveParams& prm, bool* launched) {
   return cudaErrorInvalidValue;
 }
 
+cudaError_t pcg_resident_fits(const Ctx& x, bool* fits) {
+  *fits = false;
+  if (x.g.n_sims > kMaxPersistentSims || x.g.n_cubes < 1) return cudaSuccess;
+  ResPlan P;
+  return x.solve64 ? res_plan<double>(x, &P, fits) : res_plan<float>(x, &P, fits);
+}
+
 // The on-chip PCG when the grid allows it (at most kMaxPersistentSims sims, vectors that
 // fit); *launched says whether it ran.
 cudaError_t launch_pcg_resident(const Ctx& x, const SolveParams& prm, bool* launched) {
