@@ -203,7 +203,8 @@ bcm_status bcm_step_graph(bcm_grid *grid, int n_steps, double rtol, int max_iter
  * cap on FP64 residual evaluations per solve [30]; check_every, PCG iterations
  * between two reads of the device convergence flags by the host [8];
  * barrier_timeout_s, the longest wait of a block at a grid barrier of the
- * persistent PCG before the solve gives up with BCM_E_TIMEOUT [2 s]; recycle, in
+ * persistent PCG before the solve gives up with BCM_E_TIMEOUT [2 s] (FP64 solves that take
+ * the on-chip form by default go on in two launches per iteration instead); recycle, in
  * mixed mode with the persistent PCG: 1 keeps the inner CG's search direction across
  * defect-correction cycles (the FP64 residual replaces the FP32 one: a reliable
  * update), 0 restarts the inner CG every cycle [1].  A value <= 0 keeps the current

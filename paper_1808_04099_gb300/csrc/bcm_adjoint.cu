@@ -524,7 +524,12 @@ extern "C" bcm_status bcm_adjoint_step(bcm_grid* grid, void* dev_adj, size_t byt
     if (x.auto_form) ADJ_TRY(launch_pcg_resident(x, prm, &on_chip));
     if (on_chip) {
       const bcm_status st = grid_read_err(grid);
-      if (st != BCM_OK) return st;
+      if (st != BCM_OK && st != BCM_E_TIMEOUT) return st;
+      if (st == BCM_E_TIMEOUT) {  // a wait ran out: two launches from the iterate reached
+        on_chip = false;
+        ADJ_TRY(launch_solve_begin(x));
+        ADJ_TRY(launch_residual(x, prm));
+      }
     }
     int done = 0;
     for (int it = 0; it < max_iter && !on_chip;) {

@@ -1094,10 +1094,17 @@ bcm_status solve(bcm_grid* g, double rtol, int max_iter) {
   if (g->solve64 && !mg && x.auto_form) {  // FP64 on chip where it fits, else two launches
     bool on_chip = false;
     CUDA_TRY(pcg_resident_fits(x, &on_chip));
+    if (on_chip) RUN(BCM_K_PCG, launch_pcg_resident(x, prm, &on_chip));
     if (on_chip) {
-      RUN(BCM_K_PCG, launch_pcg_resident(x, prm, &on_chip));
-      g->pcg_form = PCG_RESIDENT;
-      return read_err(g);
+      st = read_err(g);
+      if (st != BCM_E_TIMEOUT) {
+        g->pcg_form = PCG_RESIDENT;
+        return st;
+      }
+      // a wait ran out (the blocks did not run at the same time): two launches, which wait
+      // for nothing, from the iterate reached
+      RUN(BCM_K_MISC, launch_solve_begin(x));
+      RUN(BCM_K_RESIDUAL, launch_residual(x, prm));
     }
   }
   if ((st = read_flags(g, flags)) != BCM_OK) return st;

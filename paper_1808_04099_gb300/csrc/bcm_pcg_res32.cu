@@ -30,11 +30,16 @@ cudaError_t pcg_resident_fits(const Ctx& x, bool* fits) {
 }
 
 // The on-chip PCG when the grid allows it (at most kMaxPersistentSims sims, vectors that
-// fit); *launched says whether it ran.
+// fit); *launched says whether it ran.  A device that refuses the cooperative launch runs
+// another form.
 cudaError_t launch_pcg_resident(const Ctx& x, const SolveParams& prm, bool* launched) {
   *launched = false;
   if (x.g.n_sims > kMaxPersistentSims || x.g.n_cubes < 1) return cudaSuccess;
-  return x.solve64 ? launch_pcg_resident64(x, prm, launched) : res32(x, prm, launched);
+  const cudaError_t e = x.solve64 ? launch_pcg_resident64(x, prm, launched) : res32(x, prm, launched);
+  if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) return e;
+  (void)cudaGetLastError();
+  *launched = false;
+  return cudaSuccess;
 }
 
 }  // namespace bcm
