@@ -219,8 +219,9 @@ bcm_status bcm_get_solver(const bcm_grid *grid, double *inner_rtol, int32_t *max
 
 /* Launch shape of the PCG.  Until this call asks for one, a Jacobi solve whose vectors fit
  * the registers and shared memory of the GPU (grids of at most 256 sims; on 152 SMs of
- * 227 KB about 4.3M cells in FP32 inner solves and 1.6M in FP64) runs in the on-chip form
- * (bcm_stats.pcg_form 3), and larger ones persistent = 1 in mixed mode, persistent = 0 in
+ * 227 KB up to 4.36M cells in FP32 inner solves and 1.87M in FP64 on cubes of 8^3 and 16^3,
+ * 2.49M and 1.25M on cubes of 4^3) runs in the on-chip form (bcm_stats.pcg_form 3), and
+ * larger ones persistent = 1 in mixed mode, persistent = 0 in
  * FP64.  persistent = 5 (mixed mode on 16^3 cubes, grids of at most
  * 160 sims and 256 cubes per SM): one cooperative launch per solve, one block of 1024
  * threads (four x-adjacent cells of the cube in hand each) per SM,
@@ -234,8 +235,8 @@ bcm_status bcm_get_solver(const bcm_grid *grid, double *inner_rtol, int32_t *max
  * returns, as form 3 does and where the other forms launch BCM_K_ADD_CORRECTION);
  * persistent = 3: the same iteration on chip: the preconditioned residual in registers,
  * the search direction with its ghost planes in shared memory, only the cubes' face values
- * and the partial sums crossing between blocks (FP32 inner solve that fits, slabs_a = 1),
- * else the streaming form; persistent = 2:
+ * and the partial sums crossing between blocks (grids that fit, slabs_a = 1), else the
+ * streaming form; persistent = 2:
  * the single-reduction form of the iteration (Chronopoulos-Gear: one pass and one
  * barrier per iteration, three more vectors, the same iterates in exact arithmetic).
  * slabs_a = z-slabs per cube of the streaming work items (1, 2 or 4; 16^3 cubes only
@@ -245,6 +246,9 @@ bcm_status bcm_get_solver(const bcm_grid *grid, double *inner_rtol, int32_t *max
  * depend on the shape beyond rounding; bcm_stats.pcg_form says which form ran.
  * BCM_E_INVALID for other values. */
 bcm_status bcm_set_launch(bcm_grid *grid, int persistent, int slabs_a, int slabs_b);
+/* Back to the launch shape of a new grid: the on-chip form where the grid fits (the only way
+ * to ask for it in FP64), else the default of its precision. */
+bcm_status bcm_reset_launch(bcm_grid *grid);
 
 /* Test path, no GPU needed: the launch shape of the on-chip PCG (FP64 vectors, or those of
  * the FP32 inner solve) for a grid of these sizes on a device of n_sms SMs whose blocks may

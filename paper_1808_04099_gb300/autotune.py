@@ -1,6 +1,7 @@
 """Launch-shape autotuner of the PCG: the persistent cooperative solver (two passes per
-iteration streaming with 1, 2 or 4 z-slabs per work item or with its state on chip, the fused single-barrier form with bulk-copy staging, or the
-single-reduction form), or two launches per iteration with z-slabs per pass.
+iteration, with its state on chip or streaming with 1, 2 or 4 z-slabs per work item, the
+fused single-barrier form with bulk-copy staging, or the single-reduction form), or two
+launches per iteration with z-slabs per pass.
 
 Times a fixed number of PCG iterations on the grid's current right-hand side for
 every shape with the library's own CUDA-event kernel timing, restores the pressure,
@@ -17,6 +18,7 @@ from . import bcm
 # (persistent, slabs_a, slabs_b)
 SHAPES = [(5, 1, 1), (1, 1, 1), (1, 2, 1), (1, 4, 1), (3, 1, 1), (2, 1, 1), (2, 2, 1),
           (2, 4, 1), (0, 1, 1), (0, 1, 2), (0, 2, 2)]
+DEFAULT = (-1, 1, 1)  # a new grid's shape: in FP64 the only one with the state on chip
 CACHE = os.path.join(os.path.expanduser("~"), ".cache", "bcm_gb300_launch.json")
 
 
@@ -28,6 +30,14 @@ def _key(grid, device_name=None) -> str:
     shapes = ";".join(f"{pe},{sa},{sb}" for pe, sa, sb in SHAPES)
     return (f"{device_name}|B{grid.spec.B}|prec{grid.precision}|cubes{grid.spec.n_cubes}"
             f"|shapes{shapes}")
+
+
+def _set(grid, shape):
+    pe, sa, sb = shape
+    if tuple(shape) == DEFAULT:
+        grid.reset_launch()
+    else:
+        grid.set_launch(sa, sb, persistent=pe)
 
 
 def _read_cache(path: str) -> dict:
@@ -49,9 +59,9 @@ def tune(grid, iters: int = 40, use_cache: bool = True, cache_path: str | None =
     key = _key(grid, device_name) if use_cache else None
     cache = _read_cache(path) if use_cache else {}
     entry = cache.get(key)
-    if use_cache and isinstance(entry, dict) and tuple(entry.get("best", ())) in SHAPES:
-        pe, sa, sb = entry["best"]
-        grid.set_launch(sa, sb, persistent=pe)
+    if use_cache and isinstance(entry, dict) and \
+            tuple(entry.get("best", ())) in [DEFAULT, *SHAPES]:
+        _set(grid, entry["best"])
         return entry["times"]
     p = grid.field(bcm.P)
     saved = p.clone()
@@ -64,11 +74,11 @@ def tune(grid, iters: int = 40, use_cache: bool = True, cache_path: str | None =
         p.copy_(saved)
         grid.set_solver(max_cycles=caller_cycles)
     best = min(times, key=times.get)
-    pe, sa, sb = map(int, best.split(","))
-    grid.set_launch(sa, sb, persistent=pe)
+    best = tuple(map(int, best.split(",")))
+    _set(grid, best)
     if use_cache:
         cache = _read_cache(path)  # another process may have added entries meanwhile
-        cache[key] = {"best": [pe, sa, sb], "times": times}
+        cache[key] = {"best": list(best), "times": times}
         os.makedirs(os.path.dirname(os.path.abspath(path)), exist_ok=True)
         tmp = f"{path}.tmp{os.getpid()}"
         with open(tmp, "w") as f:
@@ -81,12 +91,15 @@ def _time_shapes(grid, iters, p, saved, times):
     """us per PCG iteration of every launch shape, into times.  Each includes its share
     of the defect correction's x += e (one per inner solve): the streaming form does it
     at the end of its own launch, the others in a launch of their own."""
-    for pe, sa, sb in SHAPES:
+    shapes = list(SHAPES)
+    if grid.precision == bcm.PREC_F64 and hasattr(grid, "reset_launch"):
+        shapes.append(DEFAULT)
+    for pe, sa, sb in shapes:
         if pe and sa > 1 and grid.spec.B != 16:
             continue
         if pe == 5 and (grid.spec.B != 16 or grid.precision == bcm.PREC_F64):
             continue  # the fused form runs FP32 inner solves on 16^3 cubes only
-        grid.set_launch(sa, sb, persistent=pe)
+        _set(grid, (pe, sa, sb))
         for rep in range(2):  # the first pass warms up the shape
             p.copy_(saved)
             grid.profile(True)

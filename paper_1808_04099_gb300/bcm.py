@@ -24,7 +24,7 @@ SCHEME_AB2_CENTRAL, SCHEME_QUICK_CN = 0, 1
 
 EXPORTED = ["bcm_workspace_bytes", "bcm_create_grid", "bcm_destroy_grid", "bcm_field",
             "bcm_set_geometry", "bcm_reset_time", "bcm_drag_mean", "bcm_set_solver",
-            "bcm_set_launch", "bcm_onchip_shape", "bcm_set_stencil_slabs", "bcm_get_stencil_slabs",
+            "bcm_set_launch", "bcm_reset_launch", "bcm_onchip_shape", "bcm_set_stencil_slabs", "bcm_get_stencil_slabs",
             "bcm_set_preconditioner", "bcm_apply_preconditioner",
             "bcm_set_step", "bcm_get_solver", "bcm_measure_fma_rate", "bcm_step", "bcm_step_graph", "bcm_solve_pressure",
             "bcm_adjoint_bytes", "bcm_adjoint_init", "bcm_adjoint_step",
@@ -108,6 +108,7 @@ def lib(build: bool = True):
                                        C.c_int, P]
         L.bcm_set_solver.argtypes = [P, C.c_double, C.c_int, C.c_int, C.c_double, C.c_int]
         L.bcm_set_launch.argtypes = [P, C.c_int, C.c_int, C.c_int]
+        L.bcm_reset_launch.argtypes = [P]
         L.bcm_onchip_shape.argtypes = [C.c_int] * 6 + [C.c_size_t, P]
         L.bcm_set_stencil_slabs.argtypes = [P, C.c_int]
         L.bcm_get_stencil_slabs.argtypes = [P, P]
@@ -385,11 +386,17 @@ class Grid:
     def set_launch(self, slabs_a: int = 1, slabs_b: int = 1, persistent: int = 1):
         """persistent: 0 two launches per iteration, 1 the persistent two-pass PCG
         streaming its vectors through global memory, 2 the persistent single-reduction
-        PCG, 3 the persistent two-pass PCG with its state on chip where the grid fits (the
-        default there, in FP64 too), 5 the fused single-barrier PCG (mixed
+        PCG, 3 the persistent two-pass PCG with its state on chip where the grid fits (mixed
+        precision, else the two-pass form runs), 5 the fused single-barrier PCG (mixed
         precision on 16^3 cubes, else the two-pass form runs; bool values map to 0 and
-        1)."""
+        1).  reset_launch() goes back to the default."""
         _check(lib().bcm_set_launch(self._h, int(persistent), slabs_a, slabs_b))
+
+    def reset_launch(self):
+        """The launch shape of a new grid: the PCG with its state on chip where the grid fits,
+        in FP64 too, else streaming in mixed precision and two launches per iteration in
+        FP64."""
+        _check(lib().bcm_reset_launch(self._h))
 
     def set_stencil_slabs(self, slabs: int):
         """z-slabs per 16^3 cube of the momentum and right-hand-side kernels (1, 2, 4; 0:

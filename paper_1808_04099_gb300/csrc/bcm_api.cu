@@ -646,6 +646,21 @@ extern "C" size_t bcm_workspace_bytes(const bcm_grid_desc* desc) {
   return plan(desc, T.n_slots, mg_build(desc, T), &ml).total;
 }
 
+// The PCG's launch shape of a new grid.  Measured on GB300 at 4.2M cells: the persistent
+// streaming solver is on par in FP32 and slower in FP64 (ALU-bound passes), so FP64 grids that
+// do not fit on chip run two launches per iteration.
+static void default_launch(bcm_grid* g) {
+  Ctx& x = g->ctx;
+  x.slabs_a = 1;
+  x.slabs_b = 1;
+  x.slabs_p = (g->B == 16 && g->solve64) ? 2 : 1;
+  x.persistent = (!g->solve64 && g->desc.n_sims <= 256) ? 1 : 0;
+  x.single_pass = 0;
+  x.resident = 0;
+  x.auto_form = g->desc.n_sims <= 256 ? 1 : 0;
+  x.fused = 0;  // the fused single-barrier form: selected by bcm_set_launch(5, ...)
+}
+
 extern "C" bcm_status bcm_create_grid(const bcm_grid_desc* desc, void* dev_workspace, size_t bytes,
                                       void* cuda_stream, bcm_grid** out) {
   if (!out) return fail(BCM_E_INVALID, "out is NULL");
@@ -732,16 +747,7 @@ extern "C" bcm_status bcm_create_grid(const bcm_grid_desc* desc, void* dev_works
   x.B = g->B;
   x.f64 = g->f64;
   x.solve64 = g->solve64;
-  x.slabs_a = 1;
-  x.slabs_b = 1;
-  x.slabs_p = (g->B == 16 && g->solve64) ? 2 : 1;
-  // measured on GB300 at 4.2M cells: the persistent solver is on par in FP32 and
-  // slower in FP64 (ALU-bound passes), so FP64 defaults to two launches per iteration
-  x.persistent = (!g->solve64 && desc->n_sims <= 256) ? 1 : 0;
-  x.single_pass = 0;
-  x.resident = 0;
-  x.auto_form = desc->n_sims <= 256 ? 1 : 0;
-  x.fused = 0;  // the fused single-barrier form: selected by bcm_set_launch(5, ...)
+  default_launch(g);
   x.slabs_m = 0;  // the momentum / right-hand-side slab depth: bcm_set_stencil_slabs
   x.lag_bf16 = desc->lagged_bf16;
   x.stream = s;
@@ -1607,6 +1613,12 @@ extern "C" bcm_status bcm_set_launch(bcm_grid* g, int persistent, int slabs_a, i
     g->ctx.slabs_a = slabs_a;
     g->ctx.slabs_b = slabs_b;
   }
+  return BCM_OK;
+}
+
+extern "C" bcm_status bcm_reset_launch(bcm_grid* g) {
+  if (!g) return fail(BCM_E_INVALID, "grid is NULL");
+  default_launch(g);
   return BCM_OK;
 }
 
