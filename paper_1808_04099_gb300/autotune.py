@@ -5,8 +5,8 @@ launches per iteration with z-slabs per pass.
 
 Times a fixed number of PCG iterations on the grid's current right-hand side for
 every shape with the library's own CUDA-event kernel timing, restores the pressure,
-and keeps the fastest shape.  Results are cached in a JSON file keyed by device,
-cube size, precision and cube count.
+and keeps the fastest shape.  Results are cached in a JSON file keyed by device, cube
+size, precision, numbers of cubes, sims and levels, and the revision of the kernels.
 """
 from __future__ import annotations
 
@@ -19,6 +19,7 @@ from . import bcm
 SHAPES = [(5, 1, 1), (1, 1, 1), (1, 2, 1), (1, 4, 1), (3, 1, 1), (2, 1, 1), (2, 2, 1),
           (2, 4, 1), (0, 1, 1), (0, 1, 2), (0, 2, 2)]
 DEFAULT = (-1, 1, 1)  # a new grid's shape: in FP64 the only one with the state on chip
+REVISION = 2  # of the kernels behind the shapes (2: form 3 keeps the whole state on chip)
 CACHE = os.path.join(os.path.expanduser("~"), ".cache", "bcm_gb300_launch.json")
 
 
@@ -26,10 +27,14 @@ def _key(grid, device_name=None) -> str:
     if device_name is None:
         import torch
         device_name = torch.cuda.get_device_name(grid.device)
-    # the shape list is part of the key: a cache written for other shapes is not used
+    # the shape list and the revision of the forms behind it are part of the key: a cache
+    # written for other shapes or other kernels is not used; which forms fit depends on the
+    # sims and levels too
     shapes = ";".join(f"{pe},{sa},{sb}" for pe, sa, sb in SHAPES)
-    return (f"{device_name}|B{grid.spec.B}|prec{grid.precision}|cubes{grid.spec.n_cubes}"
-            f"|shapes{shapes}")
+    sp = grid.spec
+    return (f"{device_name}|B{sp.B}|prec{grid.precision}|cubes{sp.n_cubes}"
+            f"|sims{getattr(sp, 'n_sims', 1)}|levels{getattr(sp, 'max_level', 0)}"
+            f"|rev{REVISION}|shapes{shapes}")
 
 
 def _set(grid, shape):
@@ -53,8 +58,9 @@ def tune(grid, iters: int = 40, use_cache: bool = True, cache_path: str | None =
          device_name: str | None = None) -> dict:
     """Pick and set the fastest launch shape; returns {"persistent,slabs_a,slabs_b": us
     per iteration}.  The cache (a JSON file, cache_path or CACHE) maps the device, cube
-    size, precision, cube count and shape list to the best shape and its times; an
-    unreadable cache counts as empty.  The caller's solver controls are restored."""
+    size, precision, counts (cubes, sims, levels), kernel revision and shape list to the
+    best shape and its times; an unreadable cache counts as empty.  The caller's solver
+    controls are restored."""
     path = cache_path or CACHE
     key = _key(grid, device_name) if use_cache else None
     cache = _read_cache(path) if use_cache else {}
