@@ -516,19 +516,9 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_
       st4(pb.x + base + m * BB, xv[m]);
     }
   }
-  if constexpr (FB) {
-    const TV t[1] = {rr2};
-    double val[1];
-    if constexpr (T::TPC == 32) {
-      TV w = rr2;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-      val[0] = double(w);
-    } else {
-      __shared__ double red[32];
-      block_sum_tv<T::NT, 1, TV>(t, val, red);
-    }
-    if (lt == 0) acc_add_cube(st, ACC_RR, c, val[0]);
+  if constexpr (FB) {  // (summed in FP64 from the threads on, as <r, z> below)
+    const double sum = T::sum(double(rr2));
+    if (lt == 0) acc_add_cube(st, ACC_RR, c, sum);
   }
 }
 
@@ -556,7 +546,7 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_
   poison_tile(reinterpret_cast<TV*>(smem_raw), T::CPB * T::N);
   SimState& st = g.ss[L.s];
   const bool active = valid && (mode == 2 || !st.done);
-  TV part[1] = {TV(0)};
+  TV part = TV(0);
   if (active) {
     // after a down launch with pass B (rb set) the new residual is in the buffer that
     // the iteration's parity selects, else in ra
@@ -613,21 +603,12 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_
 #pragma unroll
       for (int e = 0; e < 4; ++e) zv[e] = v[m][e] + (wl * inv[e]) * t[e];
       st4(z + base + m * BB, zv);
-      part[0] += dot4(res[m], zv);
+      part += dot4(res[m], zv);
     });
   }
   if (mode == 2 || !finest) return;
-  double val[1];
-  if constexpr (T::TPC == 32) {
-    TV w = part[0];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-    val[0] = double(w);
-  } else {
-    __shared__ double red[32];
-    block_sum_tv<T::NT, 1, TV>(part, val, red);
-  }
-  if (lt == 0 && active) acc_add_cube(st, ACC_RZ, c, val[0]);
+  const double sum = T::sum(double(part));
+  if (lt == 0 && active) acc_add_cube(st, ACC_RZ, c, sum);
 }
 
 // The decisions of an iteration (mg_decide) after the quad kernels, in a launch of one block:

@@ -134,6 +134,15 @@ struct QT {
     if constexpr (TPC == 32) __syncwarp();
     else __syncthreads();
   }
+  // sum of a cube's threads, valid in the cube's first
+  __device__ __forceinline__ static double sum(double v) {
+    if constexpr (TPC == 32) {
+      return warp_sum(v);
+    } else {
+      __shared__ double red[NT];
+      return block_sum_once<NT>(v, red);
+    }
+  }
 };
 
 // Constants of a block's cube.

@@ -181,7 +181,7 @@ __global__ __launch_bounds__(NT) void k_residual(DevGrid g, const double* __rest
 // The same on whole cubes of 16^3 or 8^3 by quad tiles (bcm_quad.cuh).  It is bound by the
 // FP64 pipe: about 10 operations a cell in the mixed mode against 22 of the padded-tile
 // kernel (the neighbour sum six instead of eleven, ||rhs|| only in a solve's first cycle,
-// the FP32 sums and diagonals in FP32): 4.2M cells in 180 us before, 128 us now.
+// each thread's FP32 sums and diagonals in FP32): 4.2M cells in 180 us before, 128 us now.
 template <int B, class TV, bool MIXED>
 __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<double>()) void k_residual_quad(
     DevGrid g, const double* __restrict__ b, const double* __restrict__ x, TV* __restrict__ r,
@@ -203,8 +203,8 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<double>()) void k
   SimState& st = g.ss[L.s];
   const bool active = valid && !(MIXED && st.outer_done);
   const bool want_bb = !MIXED || st.cycles == 0;  // (the last block counts the cycles)
-  double bb[1] = {0.0}, rr64[1] = {0.0};
-  TV rz[1] = {TV(0)}, rr[1] = {TV(0)};
+  double bb = 0.0, rr64 = 0.0;
+  TV rz = TV(0), rr = TV(0);
   if (active) {
     const int pos = lt % T::Q, i0 = (4 * pos) % B, j = (4 * pos) / B, k0 = 4 * (lt / T::Q);
     const size_t base = (size_t)c * B3 + (k0 * B + j) * B + i0;
@@ -238,39 +238,26 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<double>()) void k
       for (int q = 0; q < 4; ++q) {
         const double rhs = -V * bv[q];
         rv[q] = fma(-h, acc[q], rhs);
-        if (want_bb) bb[0] = fma(rhs, rhs, bb[0]);
+        if (want_bb) bb = fma(rhs, rhs, bb);
       }
       TV rt[4], inv[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) rt[q] = TV(rv[q]);
       quad_inv<B>(cq, i0, j, k0 + m, inv);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) rz[0] += rt[q] * (rt[q] * inv[q]);
-      rr[0] += dot4(rt, rt);
+      for (int q = 0; q < 4; ++q) rz += rt[q] * (rt[q] * inv[q]);
+      rr += dot4(rt, rt);
       st4(r + base + m * BB, rt);
       if constexpr (MIXED) {
-        rr64[0] += dot4(rv, rv);
+        rr64 += dot4(rv, rv);
         const float zero[4] = {0.f, 0.f, 0.f, 0.f};
         st4(e + base + m * BB, zero);
       }
     });
   }
-  // sums per cube (a warp, or the block)
-  auto sum = [&](auto& p) {
-    double val[1];
-    if constexpr (T::TPC == 32) {
-      auto w = p[0];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-      val[0] = double(w);
-    } else {
-      __shared__ double red[32];
-      block_sum_tv<T::NT, 1>(p, val, red);
-    }
-    return val[0];
-  };
-  const double s_rz = sum(rz), s_rr = sum(rr);
-  const double s_rr64 = MIXED ? sum(rr64) : 0.0, s_bb = want_bb ? sum(bb) : 0.0;
+  // sums per cube, in FP64 from the threads on
+  const double s_rz = T::sum(double(rz)), s_rr = T::sum(double(rr));
+  const double s_rr64 = MIXED ? T::sum(rr64) : 0.0, s_bb = want_bb ? T::sum(bb) : 0.0;
   if (lt == 0 && active) {
     if (want_bb) acc_add_cube(st, ACC_BB, c, s_bb);
     if (MIXED) acc_add_cube(st, ACC_RR64, c, s_rr64);
