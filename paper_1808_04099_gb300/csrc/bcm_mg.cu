@@ -382,9 +382,8 @@ struct PassB {
 };
 
 // alpha = <r, z> / <p, K p> of one sim (zero where the denominator is zero or not finite)
-template <class TV>
 __device__ __forceinline__ double cg_alpha_of(double rz, double pq) {
-  return pq != 0.0 && isfinite(pq) ? quick_div<TV>(rz, pq, quick_rcp<TV>(pq)) : 0.0;
+  return pq != 0.0 && isfinite(pq) ? quick_div(rz, pq, quick_rcp(pq)) : 0.0;
 }
 
 template <int B, class TV, bool FB>
@@ -446,7 +445,7 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_
     if (lt < 32) {
 #pragma unroll
       for (int o = 1; o < kStripes; o <<= 1) pq += __shfl_xor_sync(0xffffffffu, pq, o);
-      if (lt == 0) alphas[cub] = TV(cg_alpha_of<TV>(rz, pq));
+      if (lt == 0) alphas[cub] = TV(cg_alpha_of(rz, pq));
     }
   }
   T::sync();

@@ -609,7 +609,7 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
       return;
     }
     S.rr = rr;
-    S.beta = ((k == 0 && S.first) || S.rz == 0.0) ? 0.0 : quick_div<TV>(rz, S.rz, S.rrz);
+    S.beta = ((k == 0 && S.first) || S.rz == 0.0) ? 0.0 : quick_div(rz, S.rz, S.rrz);
     S.rz = rz;
   };
 
@@ -830,9 +830,9 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
       double s[1];
       words_sum<1>(va, S.cnt, s);
       // lane 0: alpha = <r, z> / <p, Kp>; lane 1: 1 / <r, z> for the next beta
-      const double d = lane == 0 ? s[0] : S.rz, y = quick_rcp<TV>(d);
+      const double d = lane == 0 ? s[0] : S.rz, y = quick_rcp(d);
       if (lane == 0) {
-        S.alpha = (d != 0.0 && isfinite(d)) ? quick_div<TV>(S.rz, d, y) : 0.0;
+        S.alpha = (d != 0.0 && isfinite(d)) ? quick_div(S.rz, d, y) : 0.0;
         if (kD && !isfinite(d)) finish(l, k, S.rr, false, true);
       }
       if (lane == 1) S.rrz = y;

@@ -15,23 +15,21 @@
 namespace bcm {
 
 // 1 / d by Newton's iteration y <- y + y (1 - d y) from the hardware's approximate
-// reciprocal (23 bits): two steps, or one (46 bits) where the quotient is then rounded to
-// FP32.  An FP64 operation takes 64 cycles on this part and the compiler's division
-// 1460; these take about 450 and 250, twice per iteration of the solver.  Exponents near
-// the ends of the range go to the division.
-template <class TV>
+// reciprocal (about 20 bits), two steps, and a quotient from it with one correction by its
+// remainder: within an ulp or so of the division's.  An FP64 operation takes 64 cycles on
+// this part and the compiler's division 1460; the reciprocal takes about 450, twice per
+// iteration of the solver.  Exponents near the ends of the range go to the division.
 __device__ __forceinline__ double quick_rcp(double d) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
   const unsigned ex = (unsigned)__double2hiint(y) >> 20 & 0x7ffu;
   if (ex - 64u > 1920u) return 1.0 / d;
   y = fma(y, fma(-d, y, 1.0), y);
-  return sizeof(TV) == 8 ? fma(y, fma(-d, y, 1.0), y) : y;
+  return fma(y, fma(-d, y, 1.0), y);
 }
-template <class TV>
 __device__ __forceinline__ double quick_div(double a, double d, double y) {  // y = 1 / d
   double q = a * y;
-  if (sizeof(TV) == 8) q = fma(fma(-d, q, a), y, q);
+  q = fma(fma(-d, q, a), y, q);
   return isfinite(q) ? q : a / d;
 }
 
