@@ -91,7 +91,14 @@ struct ResShape {
   int nls;             // sims a block may hold cells of (capacity)
   int mq;              // quads per thread whose K p / h is in shared memory (the rest: q)
   int multi;           // some block holds cells of several sims
-  int o_g, o_q, o_item, o_tab, o_sim, o_red;  // byte offsets in dynamic shared memory
+  int o_g, o_q, o_item, o_21, o_tab, o_sim, o_red;  // byte offsets in dynamic shared memory
+};
+
+// Plane entries across the item's 2:1 faces (grids of two levels): of the coarse cell at the
+// face's origin ([0]), or of the fine cells at the origin of each of its four parts (part
+// 2 h + q: the half h of its rows, the half q of each row), which lie on one plane each.
+struct ResFace21 {
+  int at[6][4];
 };
 
 // Constants of one item.
@@ -257,6 +264,29 @@ __device__ __forceinline__ TV ghost_21(const DevGrid& g, const ResShape& sh, int
   return TV(0.25) * sum;
 }
 
+// The entries of a ResFace21 for the R rows from b0 of face f of cube c.
+__device__ __forceinline__ void face_21(const DevGrid& g, const ResShape& sh, int c, int f, int b0,
+                                        int R, bool coarse, int (&at)[4]) {
+  const int d = f >> 1, B = 1 << sh.lb;
+  for (int u = 0; u < 4; ++u) at[u] = 0;
+  if (coarse) {
+    const int C = g.aux[(6 * c + f) * 4];
+    if (!bcm_expect(g, C >= 0 && C < g.n_cubes, CHK_AUX)) return;
+    const int sf = 1 << (g.max_level - g.lvl[c]), sc = 2 * sf;
+    const int A = (g.ijk[3 * c + tan1(d)] - g.ijk[3 * C + tan1(d)]) / sc;
+    const int Bb = (g.ijk[3 * c + tan2(d)] + b0 * sf - g.ijk[3 * C + tan2(d)]) / sc;
+    if (!bcm_expect(g, A >= 0 && A < B && Bb >= 0 && Bb < B, CHK_CELL)) return;
+    at[0] = face_entry(sh, C, f ^ 1, A, Bb);
+    return;
+  }
+  for (int u = 0; u < 4; ++u) {
+    const int tb = 2 * b0 + (u >> 1) * R, qb = tb >> sh.lb;
+    const int F = g.aux[(6 * c + f) * 4 + 2 * qb + (u & 1)];
+    if (bcm_expect(g, F >= 0 && F < g.n_cubes, CHK_AUX))
+      at[u] = face_entry(sh, F, f ^ 1, 0, tb - qb * B);
+  }
+}
+
 // v with its sign bit xor-ed by `sign` (an integer operation: FP64 ones are dear)
 __device__ __forceinline__ float flip(float v, unsigned sign) {
   return __uint_as_float(__float_as_uint(v) ^ sign);
@@ -276,6 +306,15 @@ __device__ __forceinline__ void ldcg4(const double* p, double (&v)[4]) {
   v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
 }
 
+__device__ __forceinline__ void ldcg2(const float* p, float (&v)[2]) {
+  const float2 t = __ldcg(reinterpret_cast<const float2*>(p));
+  v[0] = t.x; v[1] = t.y;
+}
+__device__ __forceinline__ void ldcg2(const double* p, double (&v)[2]) {
+  const double2 t = __ldcg(reinterpret_cast<const double2*>(p));
+  v[0] = t.x; v[1] = t.y;
+}
+
 // ---------------------------------------------------------------- the kernel
 //
 // M: quads per thread.  GEO: 0, or the cube edge B of whole-cube items, whose positions
@@ -289,6 +328,11 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
                                                    WordLine* __restrict__ words,
                                                    SolveParams prm, int* err) {
   constexpr bool kD = sizeof(TV) == 8;
+  // 2:1 ghosts through ResFace21, whose loads are independent, where registers are left for
+  // them (the FP64 and the largest FP32 kernels spill), else cell by cell through the cubes'
+  // tables, 4-5 us of an iteration: FP32 two-level grids of 188 cubes of 8^3 12.4 -> 8.1 us,
+  // 1648 20.0 -> 12.5, 188 of 16^3 19.2 -> 11.8 (the streaming form takes 12.1, 29.8, 19.8)
+  constexpr bool kTab = !kD && M <= 8;
   constexpr int NW = NT / 32;
   extern __shared__ __align__(16) unsigned char sm[];
   constexpr int kLb = GEO == 16 ? 4 : GEO == 8 ? 3 : 2;
@@ -301,6 +345,7 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
   TV* sg = sp + og;
   TV* sq = reinterpret_cast<TV*>(sm + sh.o_q);
   ResItem<TV>* items = reinterpret_cast<ResItem<TV>*>(sm + sh.o_item);
+  ResFace21* const f21 = reinterpret_cast<ResFace21*>(sm + sh.o_21);
   TV* tab = reinterpret_cast<TV*>(sm + sh.o_tab);
   ResSim* sims = reinterpret_cast<ResSim*>(sm + sh.o_sim);
   double* red = reinterpret_cast<double*>(sm + sh.o_red);
@@ -345,6 +390,7 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
       } else {
         I.src[f] = -1;
         fl |= (1u << 9) | (n == NB_COARSE ? 1u << (16 + f) : 1u << (24 + f));
+        if (kTab) face_21(g, sh, c, f, f < 4 ? slab * KS : 0, f < 4 ? KS : B, n == NB_COARSE, f21[it].at[f]);
       }
     }
     I.cube = c;
@@ -668,13 +714,36 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
       if (src >= 0) {
         ldcg4(fz + src + gt, zv);
       } else {
-        auto fetch = [&](int cube, int ff, int aa, int bb) {
-          return __ldcg(fz + face_entry(sh, cube, ff, aa, bb));
-        };
-        const int b = (gt >> lb) + (gf < 4 ? I.slab * KS : 0);
+        if constexpr (kTab) {
+          const int* at = f21[it].at[gf];
+          const int a = gt & (B - 1), b = gt >> lb;
+          if (I.flags >> (16 + gf) & 1u) {
+            TV w[2];
+            ldcg2(fz + at[0] + ((b >> 1) << lb) + (a >> 1), w);
+            zv[0] = zv[1] = w[0];
+            zv[2] = zv[3] = w[1];
+          } else {
+            const int lr = gf < 4 ? lk : lb, hh = b >> (lr - 1), row = (2 * b - (hh << lr)) << lb;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const int q = 2 * a + 4 * u, qa = q >> lb;
+              const TV* F = fz + at[2 * hh + qa] + row + (q - (qa << lb));
+              TV lo[4], hi[4];
+              ldcg4(F, lo);
+              ldcg4(F + B, hi);
+              zv[2 * u] = TV(0.25) * (((lo[0] + lo[1]) + hi[0]) + hi[1]);
+              zv[2 * u + 1] = TV(0.25) * (((lo[2] + lo[3]) + hi[2]) + hi[3]);
+            }
+          }
+        } else {
+          auto fetch = [&](int cube, int ff, int aa, int bb) {
+            return __ldcg(fz + face_entry(sh, cube, ff, aa, bb));
+          };
+          const int b = (gt >> lb) + (gf < 4 ? I.slab * KS : 0);
 #pragma unroll 1
-        for (int u = 0; u < 4; ++u)
-          zv[u] = ghost_21<TV>(g, sh, I.cube, gf, (gt & (B - 1)) + u, b, I.flags >> (16 + gf) & 1u, fetch);
+          for (int u = 0; u < 4; ++u)
+            zv[u] = ghost_21<TV>(g, sh, I.cube, gf, (gt & (B - 1)) + u, b, I.flags >> (16 + gf) & 1u, fetch);
+        }
       }
     };
     auto ghost_step = [&](int it, TV (&zv)[4]) {
@@ -1024,6 +1093,8 @@ bool res_shape(const Ctx& x, int nsm, size_t smem_max, ResPlan* out) {
       o += up16(E * (size_t)ipb * G);
       s.o_item = (int)o;
       o += up16(sizeof(ResItem<TV>) * (size_t)ipb);
+      s.o_21 = (int)o;
+      o += x.g.max_level && E == 4 ? up16(sizeof(ResFace21) * (size_t)ipb) : 0;
       s.o_tab = (int)o;
       o += up16(2 * E * (size_t)nls * (x.g.max_level + 1) * kW3);
       s.o_sim = (int)o;
