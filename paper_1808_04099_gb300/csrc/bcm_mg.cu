@@ -387,11 +387,11 @@ __device__ __forceinline__ double cg_alpha_of(double rz, double pq) {
 }
 
 template <int B, class TV, bool FB>
-__global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_down_quad(DevGrid g, const TV* __restrict__ r0,
+__global__ __launch_bounds__(QT<B, TV>::NT, QT<B, TV>::blocks) void k_mg_down_quad(DevGrid g, const TV* __restrict__ r0,
                                                             TV* __restrict__ r1,
                                                             TV* __restrict__ x1, int all,
                                                             PassB<TV> pb, TV wl, TV cl, int lsh) {
-  using T = QT<B>;
+  using T = QT<B, TV>;
   constexpr int B3 = T::B3, BB = T::BB, CB = B / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ CubeQ<TV> cqs[T::CPB];
@@ -403,7 +403,7 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_
   CubeQ<TV>& cq = cqs[cub];
   const bool valid = c < g.n_cubes;
   const CubeLoad L = cube_lookup(g, valid ? c : 0, lt);
-  Halo<B> H;
+  Halo<B, TV> H;
   H.lookup(g, valid ? c : 0, lt);
   cudaGridDependencySynchronize();  // launched after the previous level's kernel
   poison_tile(reinterpret_cast<TV*>(smem_raw), T::CPB * T::N);
@@ -425,16 +425,16 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_
     rout = (it & 1) ? pb.ra : pb.rb;
     pn = (it & 1) ? pb.p0 : pb.p1;
   }
-  const int pos = lt % T::Q, i0 = (4 * pos) % B, j = (4 * pos) / B, k0 = 4 * (lt / T::Q);
+  const int pos = lt % T::Q, i0 = (4 * pos) % B, j = (4 * pos) / B, k0 = T::NP * (lt / T::Q);
   const int cell0 = (k0 * B + j) * B + i0;
   const size_t base = (size_t)c * B3 + cell0;
-  TV res[4][4], v[4][4];
+  TV res[T::NP][4], v[T::NP][4];
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
+  for (int m = 0; m < T::NP; ++m) {
     ld4(r + base + m * BB, res[m]);
     if constexpr (FB) ld4(pb.q + base + m * BB, v[m]);
   }
-  TV ha[Halo<B>::R][4], hb[FB ? Halo<B>::R : 1][4];
+  TV ha[Halo<B, TV>::R][4], hb[FB ? Halo<B, TV>::R : 1][4];
   H.each(lt, [&](int u, int, int n, int cell, int stride) {
     const size_t gi = (size_t)n * B3 + cell;
     ldq(r + gi, stride, ha[u]);
@@ -467,7 +467,7 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_
   H.store(gh, g, c, lt, make, one, lsh);
   TV rr2 = TV(0);
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
+  for (int m = 0; m < T::NP; ++m) {
     if constexpr (FB) {
       axpy4(-alpha, v[m], res[m], res[m]);
       rr2 += dot4(res[m], res[m]);
@@ -485,7 +485,7 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_
                  [&](int m, const TV (&acc)[4]) { axpy4(-h, acc, res[m], res[m]); });
   // 2x2x2 sums: planes and x within the thread, y from the lane B / 4 on
 #pragma unroll
-  for (int u = 0; u < 2; ++u) {
+  for (int u = 0; u < T::NP / 2; ++u) {
     TV s0 = (res[2 * u][0] + res[2 * u][1]) + (res[2 * u + 1][0] + res[2 * u + 1][1]);
     TV s1 = (res[2 * u][2] + res[2 * u][3]) + (res[2 * u + 1][2] + res[2 * u + 1][3]);
     s0 += __shfl_xor_sync(0xffffffffu, s0, B / 4);
@@ -503,14 +503,14 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_
     }
   }
   if constexpr (FB) {  // x last: its loads would hold the registers of another block
-    TV xv[4][4], pv[4][4];
+    TV xv[T::NP][4], pv[T::NP][4];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
+    for (int m = 0; m < T::NP; ++m) {
       ld4(pb.x + base + m * BB, xv[m]);
       ld4(pn + base + m * BB, pv[m]);
     }
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
+    for (int m = 0; m < T::NP; ++m) {
       axpy4(alpha, pv[m], xv[m], xv[m]);
       st4(pb.x + base + m * BB, xv[m]);
     }
@@ -522,13 +522,13 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_
 }
 
 template <int B, class TV>
-__global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_up_quad(DevGrid g, const TV* __restrict__ ra,
+__global__ __launch_bounds__(QT<B, TV>::NT, QT<B, TV>::blocks) void k_mg_up_quad(DevGrid g, const TV* __restrict__ ra,
                                                           const TV* __restrict__ rb,
                                                           const TV* __restrict__ y1,
                                                           TV* __restrict__ z, SolveParams prm,
                                                           int mode, TV wl, TV cl, int finest,
                                                           int lsh) {
-  using T = QT<B>;
+  using T = QT<B, TV>;
   constexpr int B3 = T::B3, BB = T::BB, CB = B / 2, C3 = CB * CB * CB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ CubeQ<TV> cqs[T::CPB];
@@ -539,7 +539,7 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_
   CubeQ<TV>& cq = cqs[cub];
   const bool valid = c < g.n_cubes;
   const CubeLoad L = cube_lookup(g, valid ? c : 0, lt);
-  Halo<B> H;
+  Halo<B, TV> H;
   H.lookup(g, valid ? c : 0, lt);
   cudaGridDependencySynchronize();  // launched after the previous level's kernel
   poison_tile(reinterpret_cast<TV*>(smem_raw), T::CPB * T::N);
@@ -550,21 +550,21 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_
     // after a down launch with pass B (rb set) the new residual is in the buffer that
     // the iteration's parity selects, else in ra
     const TV* __restrict__ r = (mode == 1 && rb && !(st.iter & 1)) ? rb : ra;
-    const int pos = lt % T::Q, i0 = (4 * pos) % B, j = (4 * pos) / B, k0 = 4 * (lt / T::Q);
+    const int pos = lt % T::Q, i0 = (4 * pos) % B, j = (4 * pos) / B, k0 = T::NP * (lt / T::Q);
     const size_t base = (size_t)c * B3 + (k0 * B + j) * B + i0;
     auto coarse = [&](int cell) {
       return (((cell / BB) >> 1) * CB + (((cell / B) % B) >> 1)) * CB + ((cell % B) >> 1);
     };
-    TV res[4][4], v[4][4], yc[2][2];
+    TV res[T::NP][4], v[T::NP][4], yc[T::NP / 2][2];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) ld4(r + base + m * BB, res[m]);
+    for (int m = 0; m < T::NP; ++m) ld4(r + base + m * BB, res[m]);
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
+    for (int u = 0; u < T::NP / 2; ++u) {
       const TV* y = y1 + (size_t)c * C3 + (((k0 >> 1) + u) * CB + (j >> 1)) * CB + (i0 >> 1);
       yc[u][0] = y[0];
       yc[u][1] = y[1];
     }
-    TV ha[Halo<B>::R][4], hy[Halo<B>::R][2];
+    TV ha[Halo<B, TV>::R][4], hy[Halo<B, TV>::R][2];
     H.each(lt, [&](int u, int, int n, int cell, int stride) {
       ldq(r + (size_t)n * B3 + cell, stride, ha[u]);
       hy[u][0] = y1[(size_t)n * C3 + coarse(cell)];
@@ -585,7 +585,7 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_mg_
     };
     H.store(gh, g, c, lt, make, one, lsh);
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
+    for (int m = 0; m < T::NP; ++m) {
       TV inv[4];
       quad_inv<B>(cq, i0, j, k0 + m, inv);
       const TV ya = over * yc[m >> 1][0], yb = over * yc[m >> 1][1];
@@ -994,7 +994,7 @@ static cudaError_t up0_t(const Ctx& x, const SolveParams& prm, int mode) {
 
 template <int B, class TV>
 static cudaError_t down_quad_t(const Ctx& x, int l, int all, bool fb) {
-  using T = QT<B>;
+  using T = QT<B, TV>;
   const size_t sm = sizeof(TV) * (size_t)T::N * T::CPB;
   PassB<TV> pb{};
   if (fb) {
@@ -1017,7 +1017,7 @@ static cudaError_t down_quad_t(const Ctx& x, int l, int all, bool fb) {
 
 template <int B, class TV>
 static cudaError_t up_quad_t(const Ctx& x, int l, const SolveParams& prm, int mode, bool fb) {
-  using T = QT<B>;
+  using T = QT<B, TV>;
   const size_t sm = sizeof(TV) * (size_t)T::N * T::CPB;
   const double c4 = double(1 << (2 * l));
   auto kern = k_mg_up_quad<B, TV>;

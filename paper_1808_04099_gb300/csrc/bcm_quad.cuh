@@ -3,7 +3,7 @@
 //
 // A quad tile holds a cube's values densely (quads stay 16-byte aligned, unlike in a
 // padded tile) and its six face halos as planes of their own.  A thread owns a column of
-// four quads along z, so three of four z neighbours are registers, the x neighbours come
+// two or four quads along z, so z neighbours are registers inside it, the x neighbours come
 // from the lanes beside it, and every global load of a thread is issued before the first
 // use: the padded-tile kernels load a few cells, store them, and load again, which made
 // each cube a chain of about ten round trips to memory.
@@ -116,17 +116,21 @@ __device__ __forceinline__ void seven_point(const float (&c)[4], float xl, float
 
 // ---- the quad tile
 
-template <int B>
+// A thread's column has NP planes: two on 8^3 in FP64, where the one warp that four planes
+// leave a cube is a serial chain on one of the SM's four FP64 pipes (76 cycles an operation).
+// FP64 multigrid steps with four planes and with two: 16 cubes of 8^3 2727, 2078 us, 128
+// 3302, 2580, 1024 5658, 5373, 2880 14.1, 12.6 ms; 16 cubes of 16^3 5264, 4741 us.
+template <int B, class TT>
 struct QT {
   static constexpr int BB = B * B, B3 = B * BB, Q = BB / 4;  // quads per plane
-  static constexpr int TPC = B3 / 16;                        // threads per cube
-  static constexpr int CPB = TPC < 128 ? 128 / TPC : 1;      // cubes per block
+  static constexpr int NP = B == 8 && sizeof(TT) == 8 ? 2 : 4;
+  static constexpr int TPC = B3 / (4 * NP);                  // threads per cube
+  static constexpr int CPB = TPC == 32 ? 4 : 1;              // cubes per block
   static constexpr int NT = TPC * CPB;
   static constexpr int N = B3 + 6 * BB;                      // tile elements
   // blocks per SM that the kernels are compiled for: 768 threads in FP32, 512 in FP64 (whose
   // passes are bound by the FP64 pipe)
-  template <class TV>
-  static constexpr int blocks() { return (sizeof(TV) == 4 ? 768 : 512) / NT; }
+  static constexpr int blocks = (sizeof(TT) == 4 ? 768 : 512) / NT;
   // threads of one cube: a warp or the block
   __device__ __forceinline__ static void sync() {
     if constexpr (TPC == 32) __syncwarp();
@@ -158,7 +162,7 @@ struct CubeQ {
 
 // The constants of cube c, loaded by the 32 first threads of the cube (lt: thread within the
 // cube) in two steps, so that the table lookups of the first are in flight together with a
-// kernel's own first loads; QT<B>::sync() publishes them.  Only tables that no kernel
+// kernel's own first loads; QT::sync() publishes them.  Only tables that no kernel
 // writes are read.
 struct CubeLoad {
   int n, w, e0, e1, s, lv;
@@ -257,9 +261,9 @@ __device__ __forceinline__ void ldq(const TV* __restrict__ p, int stride, TV (&v
 // The tile's halo planes, each thread R quads of them, in two steps: the neighbour ids are
 // looked up with the cube's other constants, so a kernel issues its halo loads together
 // with those of its own cells, and forms the halo values once the constants are there.
-template <int B>
+template <int B, class TT>
 struct Halo {
-  using T = QT<B>;
+  using T = QT<B, TT>;
   static constexpr int R = (6 * T::Q + T::TPC - 1) / T::TPC;
   int n[R];
   __device__ __forceinline__ void lookup(const DevGrid& g, int c, int lt) {
@@ -324,20 +328,20 @@ __device__ __forceinline__ void own_quad(TV* __restrict__ S, TV* __restrict__ gh
   }
 }
 
-// The 7-point sums (K v / h) of a thread's column of four quads, planes k0 .. k0 + 3, from
+// The 7-point sums (K v / h) of a thread's column of NP quads, planes k0 .. k0 + NP - 1, from
 // the complete tile; out(m, acc) consumes plane k0 + m.  The threads of a warp call it
 // together.
-template <int B, class TV, class CQ, class Out>
+template <int B, class TV, int NP, class CQ, class Out>
 __device__ __forceinline__ void quad_column(const TV* __restrict__ S, const TV* __restrict__ gh,
                                             const CQ& cq, int i0, int j, int k0,
-                                            const TV (&v)[4][4], const Out& out) {
+                                            const TV (&v)[NP][4], const Out& out) {
   constexpr int BB = B * B;
   TV zm[4], zp[4];
   const int o = (k0 * B + j) * B + i0;
   ld4(k0 > 0 ? S + o - BB : gh + 4 * BB + j * B + i0, zm);
-  ld4(k0 < B - 4 ? S + o + 4 * BB : gh + 5 * BB + j * B + i0, zp);
+  ld4(k0 < B - NP ? S + o + NP * BB : gh + 5 * BB + j * B + i0, zp);
 #pragma unroll
-  for (int m = 0; m < 4; ++m) {
+  for (int m = 0; m < NP; ++m) {
     const int kk = k0 + m, om = o + m * BB;
     TV ym[4], yp[4], acc[4];
     ld4(j > 0 ? S + om - B : gh + 2 * BB + kk * B + i0, ym);
@@ -350,7 +354,7 @@ __device__ __forceinline__ void quad_column(const TV* __restrict__ S, const TV* 
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       b[e] = m == 0 ? zm[e] : v[m > 0 ? m - 1 : 0][e];
-      t[e] = m == 3 ? zp[e] : v[m < 3 ? m + 1 : 3][e];
+      t[e] = m == NP - 1 ? zp[e] : v[m < NP - 1 ? m + 1 : m][e];
     }
     seven_point(v[m], xl, xh, ym, yp, b, t, acc);
     if (cq.c21) {  // 2:1 faces: weight 2/3 on the fine side, 4/3 on the coarse (R7)

@@ -183,10 +183,10 @@ __global__ __launch_bounds__(NT) void k_residual(DevGrid g, const double* __rest
 // kernel (the neighbour sum six instead of eleven, ||rhs|| only in a solve's first cycle,
 // each thread's FP32 sums and diagonals in FP32): 4.2M cells in 180 us before, 128 us now.
 template <int B, class TV, bool MIXED>
-__global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<double>()) void k_residual_quad(
+__global__ __launch_bounds__(QT<B, double>::NT, QT<B, double>::blocks) void k_residual_quad(
     DevGrid g, const double* __restrict__ b, const double* __restrict__ x, TV* __restrict__ r,
     float* __restrict__ e, SolveParams prm) {
-  using T = QT<B>;
+  using T = QT<B, double>;
   constexpr int B3 = T::B3, BB = T::BB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ CubeQ<TV> cqs[T::CPB];
@@ -197,7 +197,7 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<double>()) void k
   CubeQ<TV>& cq = cqs[cub];
   const bool valid = c < g.n_cubes;
   const CubeLoad L = cube_lookup(g, valid ? c : 0, lt);
-  Halo<B> H;
+  Halo<B, double> H;
   H.lookup(g, valid ? c : 0, lt);
   poison_tile(reinterpret_cast<double*>(smem_raw), T::CPB * T::N);
   SimState& st = g.ss[L.s];
@@ -206,11 +206,11 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<double>()) void k
   double bb = 0.0, rr64 = 0.0;
   TV rz = TV(0), rr = TV(0);
   if (active) {
-    const int pos = lt % T::Q, i0 = (4 * pos) % B, j = (4 * pos) / B, k0 = 4 * (lt / T::Q);
+    const int pos = lt % T::Q, i0 = (4 * pos) % B, j = (4 * pos) / B, k0 = T::NP * (lt / T::Q);
     const size_t base = (size_t)c * B3 + (k0 * B + j) * B + i0;
-    double v[4][4], ha[Halo<B>::R][4];
+    double v[T::NP][4], ha[Halo<B, double>::R][4];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) ld4(x + base + m * BB, v[m]);
+    for (int m = 0; m < T::NP; ++m) ld4(x + base + m * BB, v[m]);
     H.each(lt, [&](int u, int, int n, int cell, int stride) {
       ldq(x + (size_t)n * B3 + cell, stride, ha[u]);
     });
@@ -223,7 +223,7 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<double>()) void k
     auto one = [&](int n, int cell) { return x[(size_t)n * B3 + cell]; };
     H.store(gh, g, c, lt, make, one, 0);
 #pragma unroll
-    for (int m = 0; m < 4; ++m) own_quad<B>(S, gh, cq, i0, j, k0 + m, v[m]);
+    for (int m = 0; m < T::NP; ++m) own_quad<B>(S, gh, cq, i0, j, k0 + m, v[m]);
     T::sync();
     const double h0 = g.sp[L.s].h0, h = g.max_level && g.lvl[c] ? 0.5 * h0 : h0;
     const double V = h * h * h, mean = st.bmean;
@@ -371,10 +371,10 @@ __global__ __launch_bounds__(NT) void k_cg_a(DevGrid g, const TV* __restrict__ r
 // comes from the multigrid V-cycle, else it is r / diag.
 // ===========================================================================
 template <int B, class TV, bool Z>
-__global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_cg_a_quad(DevGrid g, const TV* __restrict__ r,
+__global__ __launch_bounds__(QT<B, TV>::NT, QT<B, TV>::blocks) void k_cg_a_quad(DevGrid g, const TV* __restrict__ r,
                                                          TV* __restrict__ p0, TV* __restrict__ p1,
                                                          TV* __restrict__ q) {
-  using T = QT<B>;
+  using T = QT<B, TV>;
   constexpr int B3 = T::B3, BB = T::BB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ CubeQ<TV> cqs[T::CPB];
@@ -385,7 +385,7 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_cg_
   CubeQ<TV>& cq = cqs[cub];
   const bool valid = c < g.n_cubes;
   const CubeLoad L = cube_lookup(g, valid ? c : 0, lt);
-  Halo<B> H;
+  Halo<B, TV> H;
   H.lookup(g, valid ? c : 0, lt);
   cudaGridDependencySynchronize();  // (multigrid iteration: launched while the V-cycle drains)
   poison_tile(reinterpret_cast<TV*>(smem_raw), T::CPB * T::N);
@@ -398,15 +398,15 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_cg_
     TV* __restrict__ pnew = (it & 1) ? p0 : p1;
     const TV beta = TV(st.beta);
     const bool first = it == 0;
-    const int pos = lt % T::Q, i0 = (4 * pos) % B, j = (4 * pos) / B, k0 = 4 * (lt / T::Q);
+    const int pos = lt % T::Q, i0 = (4 * pos) % B, j = (4 * pos) / B, k0 = T::NP * (lt / T::Q);
     const size_t base = (size_t)c * B3 + (k0 * B + j) * B + i0;
-    TV v[4][4], pp[4][4];
+    TV v[T::NP][4], pp[T::NP][4];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
+    for (int m = 0; m < T::NP; ++m) {
       ld4(r + base + m * BB, v[m]);
       if (!first) ld4(pold + base + m * BB, pp[m]);
     }
-    TV ha[Halo<B>::R][4], hb[Halo<B>::R][4];
+    TV ha[Halo<B, TV>::R][4], hb[Halo<B, TV>::R][4];
     H.each(lt, [&](int u, int, int n, int cell, int stride) {
       const size_t gi = (size_t)n * B3 + cell;
       ldq(r + gi, stride, ha[u]);
@@ -434,7 +434,7 @@ __global__ __launch_bounds__(QT<B>::NT, QT<B>::template blocks<TV>()) void k_cg_
     };
     H.store(gh, g, c, lt, make, one, 0);
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
+    for (int m = 0; m < T::NP; ++m) {
       if constexpr (!Z) {
         TV inv[4];
         quad_inv<B>(cq, i0, j, k0 + m, inv);
@@ -736,7 +736,7 @@ static cudaError_t allow_smem(K kernel, size_t bytes) {
 
 template <int B, class TV, bool MIXED>
 static cudaError_t residual_quad_t(const Ctx& x, const SolveParams& prm) {
-  using T = QT<B>;
+  using T = QT<B, double>;
   const size_t sm = sizeof(double) * (size_t)T::N * T::CPB;
   auto kern = k_residual_quad<B, TV, MIXED>;
   cudaError_t e = allow_dynamic_smem(kern, sm);
@@ -772,7 +772,7 @@ cudaError_t launch_residual(const Ctx& x, const SolveParams& prm) {
 
 template <int B, class TV>
 static cudaError_t cg_a_quad_t(const Ctx& x, const SolveParams& prm) {
-  using T = QT<B>;
+  using T = QT<B, TV>;
   const size_t sm = sizeof(TV) * (size_t)T::N * T::CPB;
   auto kern = prm.mg ? k_cg_a_quad<B, TV, true> : k_cg_a_quad<B, TV, false>;
   cudaError_t e = allow_dynamic_smem(kern, sm);
