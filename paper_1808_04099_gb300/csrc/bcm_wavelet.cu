@@ -55,8 +55,19 @@ __device__ __forceinline__ int line_at(int d, int a, int b, int pos) {
 // so x - (p + q) / 2 as one fused operation rounds as the separate product and difference
 // do, and at the ends (p + p) / 2 is p: 2 FP64 operations a value instead of 3 (the passes
 // are bound by the FP64 pipe: on 4.2M cells the forward kernel takes 100 us, 191 with the
-// divisions of the quantizer and run-time lines; decoding 150 us, 165 before).
-template <int B, int M>
+// divisions of the quantizer and run-time lines; decoding 150 us, 165 before).  That holds
+// away from the ends of the range: with steps near them (wav_inv) values may be subnormal,
+// whose halves round, or p + p overflow, and SEP takes the separate operations.
+template <bool SEP>
+__device__ __forceinline__ double lift_add(double x, double c, double s) {  // x + c s
+  return SEP ? __dadd_rn(x, __dmul_rn(c, s)) : __fma_rn(c, s, x);
+}
+// x + c (p + p), c2 = 2 c
+template <bool SEP>
+__device__ __forceinline__ double lift_end(double x, double c, double c2, double p) {
+  return SEP ? __dadd_rn(x, __dmul_rn(c, __dadd_rn(p, p))) : __fma_rn(c2, p, x);
+}
+template <int B, int M, bool SEP>
 __device__ __forceinline__ void lift_forward(double* X, int d, int a, int b) {
   constexpr int H = M / 2;
   double x[M], dt[H];
@@ -64,17 +75,17 @@ __device__ __forceinline__ void lift_forward(double* X, int d, int a, int b) {
   for (int i = 0; i < M; ++i) x[i] = X[line_at<B>(d, a, b, i)];
 #pragma unroll
   for (int i = 0; i < H; ++i)
-    dt[i] = i + 1 < H ? __fma_rn(-0.5, __dadd_rn(x[2 * i], x[i + 1 < H ? 2 * i + 2 : 0]), x[2 * i + 1])
-                      : __dsub_rn(x[2 * i + 1], x[2 * i]);
+    dt[i] = i + 1 < H ? lift_add<SEP>(x[2 * i + 1], -0.5, __dadd_rn(x[2 * i], x[i + 1 < H ? 2 * i + 2 : 0]))
+                      : lift_end<SEP>(x[2 * i + 1], -0.5, -1.0, x[2 * i]);
 #pragma unroll
   for (int i = 0; i < H; ++i) {
-    X[line_at<B>(d, a, b, i)] = i > 0 ? __fma_rn(0.25, __dadd_rn(dt[i > 0 ? i - 1 : 0], dt[i]), x[2 * i])
-                                      : __fma_rn(0.5, dt[0], x[0]);
+    X[line_at<B>(d, a, b, i)] = i > 0 ? lift_add<SEP>(x[2 * i], 0.25, __dadd_rn(dt[i > 0 ? i - 1 : 0], dt[i]))
+                                      : lift_end<SEP>(x[0], 0.25, 0.5, dt[0]);
     X[line_at<B>(d, a, b, H + i)] = dt[i];
   }
 }
 
-template <int B, int M>
+template <int B, int M, bool SEP>
 __device__ __forceinline__ void lift_inverse(double* X, int d, int a, int b) {
   constexpr int H = M / 2;
   double e[H], dt[H];
@@ -85,36 +96,36 @@ __device__ __forceinline__ void lift_inverse(double* X, int d, int a, int b) {
   }
 #pragma unroll
   for (int i = 0; i < H; ++i)
-    e[i] = i > 0 ? __fma_rn(-0.25, __dadd_rn(dt[i > 0 ? i - 1 : 0], dt[i]), e[i])
-                 : __fma_rn(-0.5, dt[0], e[0]);
+    e[i] = i > 0 ? lift_add<SEP>(e[i], -0.25, __dadd_rn(dt[i > 0 ? i - 1 : 0], dt[i]))
+                 : lift_end<SEP>(e[0], -0.25, -0.5, dt[0]);
 #pragma unroll
   for (int i = 0; i < H; ++i) {
     X[line_at<B>(d, a, b, 2 * i)] = e[i];
     X[line_at<B>(d, a, b, 2 * i + 1)] =
-        i + 1 < H ? __fma_rn(0.5, __dadd_rn(e[i], e[i + 1 < H ? i + 1 : 0]), dt[i])
-                  : __dadd_rn(dt[i], e[i]);
+        i + 1 < H ? lift_add<SEP>(dt[i], 0.5, __dadd_rn(e[i], e[i + 1 < H ? i + 1 : 0]))
+                  : lift_end<SEP>(dt[i], 0.5, 1.0, e[i]);
   }
 }
 
 // the levels M = B, B/2, ..., 2 forward, and back
-template <int B, int M>
+template <int B, int M, bool SEP>
 __device__ __forceinline__ void wav_forward(double* X) {
   if constexpr (M >= 2) {
 #pragma unroll 1
     for (int d = 0; d < 3; ++d) {
-      if (threadIdx.x < M * M) lift_forward<B, M>(X, d, threadIdx.x % M, threadIdx.x / M);
+      if (threadIdx.x < M * M) lift_forward<B, M, SEP>(X, d, threadIdx.x % M, threadIdx.x / M);
       __syncthreads();
     }
-    wav_forward<B, M / 2>(X);
+    wav_forward<B, M / 2, SEP>(X);
   }
 }
-template <int B, int M>
+template <int B, int M, bool SEP>
 __device__ __forceinline__ void wav_inverse(double* X) {
   if constexpr (M >= 2) {
-    wav_inverse<B, M / 2>(X);
+    wav_inverse<B, M / 2, SEP>(X);
 #pragma unroll 1
     for (int d = 2; d >= 0; --d) {
-      if (threadIdx.x < M * M) lift_inverse<B, M>(X, d, threadIdx.x % M, threadIdx.x / M);
+      if (threadIdx.x < M * M) lift_inverse<B, M, SEP>(X, d, threadIdx.x % M, threadIdx.x / M);
       __syncthreads();
     }
   }
@@ -122,7 +133,7 @@ __device__ __forceinline__ void wav_inverse(double* X) {
 
 // rint(c / step) as an integer, |result| < 2^30, or *bad.  With y = 1 / step rounded,
 // t = c y is within 2^-51 |t| of the rounded quotient, so below 2^29 both round to the same
-// integer unless t lies within 2^-20 of a half-integer; only then, and when y is not
+// integer unless t lies within 2^-19 of a half-integer; only then, and when y is not
 // finite (wav_inv), the quotient itself is formed (a division costs about 20 FP64
 // operations, this 4: adding 3 2^51 leaves the rounded integer in the low word).
 __device__ __forceinline__ int32_t quantize(double c, double step, double y, bool* bad) {
@@ -130,7 +141,7 @@ __device__ __forceinline__ int32_t quantize(double c, double step, double y, boo
   const double t = __dmul_rn(c, y), m = __dadd_rn(t, kMagic52);
   const double off = __dsub_rn(t, __dsub_rn(m, kMagic52));
   const int ht = __double2hiint(t) & 0x7fffffff, ho = __double2hiint(off) & 0x7fffffff;
-  // 0x41c00000: 2^29; 0x3fdffff8: 0.5 - 2^-20
+  // 0x41c00000: 2^29; 0x3fdffff8: 0.5 - 2^-19
   if (ht < 0x41c00000 && ho < 0x3fdffff8) return __double2loint(m);
   const double r = rint(__ddiv_rn(c, step));
   if (!(fabs(r) < 1073741824.0)) {
@@ -139,7 +150,8 @@ __device__ __forceinline__ int32_t quantize(double c, double step, double y, boo
   }
   return (int32_t)r;
 }
-// 1 / step for quantize, NaN (every value takes the quotient) near the ends of the range
+// 1 / step for quantize, NaN (every value takes the quotient, the transforms the separate
+// operations) near the ends of the range
 inline double wav_inv(double step) { return step > 1e-280 && step < 1e280 ? 1.0 / step : NAN; }
 
 __device__ __forceinline__ uint32_t zigzag(int32_t q) {
@@ -171,7 +183,7 @@ __device__ __forceinline__ unsigned long long block_sum_u64(unsigned long long v
 }
 
 // forward transform, quantization, Rice parameter and record size of one cube
-template <int B, class T>
+template <int B, class T, bool SEP>
 __global__ __launch_bounds__(B * B) void k_wav_forward(const T* __restrict__ f, double step,
                                                        double inv,
                                                        uint32_t* __restrict__ zc,
@@ -186,7 +198,7 @@ __global__ __launch_bounds__(B * B) void k_wav_forward(const T* __restrict__ f, 
   for (int q = threadIdx.x; q < B3; q += NT)
     X[tix<B>(q % B, (q / B) % B, q / (B * B))] = double(f[(size_t)c * B3 + q]);
   __syncthreads();
-  wav_forward<B, B>(X);
+  wav_forward<B, B, SEP>(X);
   unsigned long long zsum = 0;
   bool bad = false;
   uint32_t zq[B3 / NT];
@@ -409,7 +421,7 @@ __device__ __forceinline__ void rice_warp_entries(const uint32_t* W, int k, uint
 // codes past the B^3-th are ignored, and a record whose B^3 codes do not fit in its bit
 // count is malformed (error bit 2, its values from the first code that does not fit
 // are 0).
-template <int B, class T>
+template <int B, class T, bool SEP>
 __global__ __launch_bounds__(B * B) void k_wav_decode(const uint32_t* __restrict__ in,
                                                       const uint32_t* __restrict__ off,
                                                       size_t words, uint32_t wcap, double step,
@@ -487,7 +499,7 @@ __global__ __launch_bounds__(B * B) void k_wav_decode(const uint32_t* __restrict
   }
   if (t == 0 && valid < (uint32_t)B3) atomicOr(err, 2);
   __syncthreads();
-  wav_inverse<B, B>(X);
+  wav_inverse<B, B, SEP>(X);
   for (int q = threadIdx.x; q < B3; q += NT)
     f[(size_t)c * B3 + q] = T(X[tix<B>(q % B, (q / B) % B, q / (B * B))]);
 }
@@ -508,10 +520,11 @@ cudaError_t wav_allow(K kern, size_t bytes) {
 template <int B, class T>
 cudaError_t compress_t(const Ctx& x, const void* field, double step, uint32_t* zc,
                        uint32_t* cube_nbits, uint32_t* cube_k, uint32_t* off, int* err) {
-  auto kf = k_wav_forward<B, T>;
+  const double inv = wav_inv(step);
+  auto kf = std::isnan(inv) ? k_wav_forward<B, T, true> : k_wav_forward<B, T, false>;
   cudaError_t e = wav_allow(kf, wav_smem<B>());
   if (e != cudaSuccess) return e;
-  kf<<<x.g.n_cubes, B * B, wav_smem<B>(), x.stream>>>((const T*)field, step, wav_inv(step), zc,
+  kf<<<x.g.n_cubes, B * B, wav_smem<B>(), x.stream>>>((const T*)field, step, inv, zc,
                                                       cube_nbits, cube_k, err);
   k_wav_offsets<<<1, 1024, 0, x.stream>>>(cube_nbits, nullptr, x.g.n_cubes, off);
   return cudaGetLastError();
@@ -521,7 +534,7 @@ template <int B, class T>
 cudaError_t decompress_t(const Ctx& x, void* field, const uint32_t* in, size_t words,
                          uint32_t max_payload, double step, uint32_t* off, int* err) {
   k_wav_offsets<<<1, 1024, 0, x.stream>>>(nullptr, in + kHead, x.g.n_cubes, off);
-  auto kd = k_wav_decode<B, T>;
+  auto kd = std::isnan(wav_inv(step)) ? k_wav_decode<B, T, true> : k_wav_decode<B, T, false>;
   const uint32_t wcap = std::min<uint32_t>(max_payload, 48u * B * B * B / 32u);
   const size_t sm = wav_dec_smem<B>(wcap);
   cudaError_t e = wav_allow(kd, sm);
