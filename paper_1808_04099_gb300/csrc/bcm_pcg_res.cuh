@@ -5,16 +5,21 @@
 // Work items are z-slabs of cubes; block p owns a contiguous run of them (the paper's
 // load-balanced linear distribution, Eq. loaddist), which is a contiguous range of the
 // cube-major vectors.  Thread t keeps the quads (four cells along x) t, t + NT, ... of
-// the range: z = M^-1 r in registers (r itself is never stored: its recurrence scaled by
-// the diagonal is z -= alpha M^-1 q), the iterate x in registers where they suffice, the
-// search direction p and K p / h in shared memory.  A cell's neighbours in other items
-// are six ghost planes per item in shared memory, which hold the neighbours' p and are
+// the range: in FP64 z = M^-1 r in registers (r itself is never stored: its recurrence scaled
+// by the diagonal is z -= alpha M^-1 q), in FP32 r; the iterate x in registers where they
+// suffice, the search direction p and K p / h in shared memory.  FP32 takes alpha over
+// <p, K p> / h0 and adds up h0 x, so that one rounded factor steps both x and r: with z's
+// factor rounded apart from x's, and r formed back from z in the sums, errors of one sign in
+// all cells left a smooth error in the pressure that later iterations do not see (relative
+// error at rtol 1e-12 on 246k cells 5.2e-13, now 1.6e-13; streaming form 1.4e-13).
+// A cell's neighbours in other items are six ghost planes per item in shared memory, which
+// hold the neighbours' p and are
 // advanced by the same recurrence p = z + beta p as the cells themselves, so the only
 // values that cross between blocks are the z of the items' face cells (fz, one plane per
 // face, in L2).  An iteration is
 //   pass A  p = z + beta p on the cells and the ghost planes; K p; <p, Kp>
 //   wait for <p, Kp> of every block of the sim -> alpha
-//   pass B  z -= alpha M^-1 K p, x += alpha p; face z out; <r, z>, <r, r>
+//   pass B  r (or z) -= alpha (M^-1) K p, x += alpha p; face z out; <r, z>, <r, r>
 //   wait for <r, z>, <r, r> of every block of the sim -> beta, convergence.
 //
 // There is no grid barrier.  A block publishes each partial sum as one 16-byte word with
@@ -111,12 +116,14 @@ struct ResItem {
   unsigned w3;      // Jacobi face weights of the slab (3 bits each)
   unsigned flags;   // bit f: face f is a domain outflow (ghost -p); bits 8, 9, 10:
                     // some weight is not 3, some face is 2:1, an x face's weight is not 3; bits 16 + f / 24 + f: coarse, fine
-  TV h, inv, dia;   // cell size, 1/diag and diag of a cell without special faces
+  TV h, inv, dia;   // cell size (FP32: over the sim's h0), 1/diag and diag of a cell without
+                    // special faces
 };
 
 struct ResSim {
   double alpha, beta, rz, rrz;  // rrz = 1 / rz
   double rz0, rr, tol2;         // <r, z> at entry, <r, r> of the last decision, the target
+  double ih0;                   // 1 / h0
   int kdone;           // iterations this launch ran
   int done, first;
   int e0, cnt;         // the sim's words: first index and number of blocks
@@ -399,7 +406,7 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
     I.tab = ((s - sim_lo) * (g.max_level + 1) + lv) * kW3;
     I.w3 = w3;
     I.flags = fl;
-    I.h = TV(P0.h0 / double(1 << lv));
+    I.h = TV((kD ? P0.h0 : 1.0) / double(1 << lv));
     I.inv = TV(P0.invdiag[lv][18]);
     I.dia = TV(1) / I.inv;
   }
@@ -420,6 +427,7 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
     S.rr = st.rr;
     S.tol2 = inner ? st.inner_tol2 : st.tol2;
     S.rrz = S.rz != 0.0 ? 1.0 / S.rz : 0.0;
+    S.ih0 = 1.0 / g.sp[s].h0;
     S.done = st.done ? 1 : 0;
     S.kdone = 0;
     S.first = cont ? 0 : 1;
@@ -494,11 +502,21 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
     if (kk == 0) st4(F + 4 * FX + (j << lb) + i0, zv);
     if (kk == KS - 1) st4(F + 4 * FX + BB + (j << lb) + i0, zv);
   };
+  // 1 / diag of the four cells of a quad
+  auto quad_invs = [&](const ResItem<TV>& I, int i0, int j, int kk, TV (&iv)[4]) {
+    if (I.flags >> 8 & 1u) {
+      const unsigned v = s3q(I, i0, j, kk);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) iv[e] = tab[I.tab + (int)(v >> (8 * e) & 255u)];
+    } else {
+      iv[0] = iv[1] = iv[2] = iv[3] = I.inv;
+    }
+  };
   auto live = [&](int it) { return !multi || !sims[items[it].sim].done; };
   auto sim_at = [&](int it) -> const ResSim& { return sims[multi ? items[it].sim : 0]; };
 
   // ---- state at entry
-  TV z[M][4];
+  TV z[M][4];  // FP64: z; FP32: r
   TV xr[XR ? M : 1][4];
   TV qr[MQR ? MQR : 1][4];
 #pragma unroll
@@ -514,11 +532,15 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
       if (inner) xr[m][0] = xr[m][1] = xr[m][2] = xr[m][3] = TV(0);
       else ld4(x + base + c0, xr[m]);
     }
-    const unsigned v = (I.flags >> 8 & 1u) ? s3q(I, i0, j, kk) : 0x12121212u;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) z[m][e] = rv[e] * tab[I.tab + (int)(v >> (8 * e) & 255u)];
     st4(sp + c0, pv);
-    put_faces(it, i0, j, kk, z[m]);
+    TV iv[4], zv[4];
+    quad_invs(I, i0, j, kk, iv);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      zv[e] = rv[e] * iv[e];
+      z[m][e] = kD ? zv[e] : rv[e];
+    }
+    put_faces(it, i0, j, kk, zv);
   }
   // face f and position t on it of entry o of an item's planes
   auto plane = [&](int o, int& f, int& t) {
@@ -789,7 +811,14 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
       TV pv[4];
       const int c0 = cell0(it, i0, j, kk);
       ld4(sp + c0, pv);
-      axpy4(beta, pv, z[m], pv);
+      if constexpr (kD) {
+        axpy4(beta, pv, z[m], pv);
+      } else {
+        TV iv[4];
+        quad_invs(items[it], i0, j, kk, iv);
+        mul4(z[m], iv, iv);
+        axpy4(beta, pv, iv, pv);
+      }
       st4(sp + c0, pv);
     }
     __syncthreads();
@@ -933,7 +962,7 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
       break;
     }
     if (kD && !multi && sims[0].done) break;
-    // ---- pass B: z -= alpha M^-1 K p, face planes, <r, z>, <r, r>
+    // ---- pass B: the residual's step, face planes, <r, z>, <r, r>
     TV rs[2] = {TV(0), TV(0)};
     const int tid_b = opaque();
 #pragma unroll
@@ -952,26 +981,36 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
           for (int e = 0; e < 4; ++e) acc[e] = qr[m - (M - MQR) > 0 ? m - (M - MQR) : 0][e];
         }
         const TV ah = TV(sim_at(it).alpha) * I.h;
-        // one diagonal value in the quad (bar its ends in a cube at an x domain face)
-        const unsigned v4 = (I.flags >> 8 & 1u) ? s3q(I, i0, j, kk) : 0x12121212u;
-        const int w = I.tab + (int)(v4 >> 8 & 255u);
-        const TV t = ah * tab[w], dia = tab[ntab + w];
-        if (!(I.flags >> 10 & 1u)) {
-          axpy4(-t, acc, z[m], z[m]);
-          rz = dot4(z[m], z[m]) * dia;
-          rr = rz * dia;
+        if constexpr (kD) {
+          // one diagonal value in the quad (bar its ends in a cube at an x domain face)
+          const unsigned v4 = (I.flags >> 8 & 1u) ? s3q(I, i0, j, kk) : 0x12121212u;
+          const int w = I.tab + (int)(v4 >> 8 & 255u);
+          const TV t = ah * tab[w], dia = tab[ntab + w];
+          if (!(I.flags >> 10 & 1u)) {
+            axpy4(-t, acc, z[m], z[m]);
+            rz = dot4(z[m], z[m]) * dia;
+            rr = rz * dia;
+          } else {
+            const int w0 = I.tab + (int)(v4 & 255u), w1 = I.tab + (int)(v4 >> 24);
+            z[m][0] -= ah * tab[w0] * acc[0];
+            z[m][1] -= t * acc[1];
+            z[m][2] -= t * acc[2];
+            z[m][3] -= ah * tab[w1] * acc[3];
+            const TV r0 = z[m][0] * tab[ntab + w0], r3 = z[m][3] * tab[ntab + w1];
+            const TV r12 = (z[m][1] * z[m][1] + z[m][2] * z[m][2]) * dia;
+            rz = z[m][0] * r0 + (z[m][3] * r3 + r12);
+            rr = r0 * r0 + (r3 * r3 + r12 * dia);
+          }
+          put_faces(it, i0, j, kk, z[m]);
         } else {
-          const int w0 = I.tab + (int)(v4 & 255u), w1 = I.tab + (int)(v4 >> 24);
-          z[m][0] -= ah * tab[w0] * acc[0];
-          z[m][1] -= t * acc[1];
-          z[m][2] -= t * acc[2];
-          z[m][3] -= ah * tab[w1] * acc[3];
-          const TV r0 = z[m][0] * tab[ntab + w0], r3 = z[m][3] * tab[ntab + w1];
-          const TV r12 = (z[m][1] * z[m][1] + z[m][2] * z[m][2]) * dia;
-          rz = z[m][0] * r0 + (z[m][3] * r3 + r12);
-          rr = r0 * r0 + (r3 * r3 + r12 * dia);
+          TV zv[4];
+          quad_invs(I, i0, j, kk, zv);
+          axpy4(-ah, acc, z[m], z[m]);
+          mul4(z[m], zv, zv);
+          rz = dot4(z[m], zv);
+          rr = dot4(z[m], z[m]);
+          put_faces(it, i0, j, kk, zv);
         }
-        put_faces(it, i0, j, kk, z[m]);
       }
       if (multi) {
         unit_sum(cell0(it, i0, j, kk) >> 6, 0, rz);
@@ -1028,7 +1067,7 @@ __global__ __launch_bounds__(NT, 1) void k_pcg_res(DevGrid g, ResShape sh, TV* _
         double x64[4];
         ld4(prm.x64_add + gi, x64);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) x64[e] += double(xv[e]);
+        for (int e = 0; e < 4; ++e) x64[e] = fma(double(xv[e]), sim_at(it).ih0, x64[e]);
         st4(prm.x64_add + gi, x64);
       }
       TV pv[4];

@@ -72,6 +72,17 @@ __device__ __forceinline__ void axpy4(double a, const double (&x)[4], const doub
 #pragma unroll
   for (int e = 0; e < 4; ++e) out[e] = fma(a, x[e], y[e]);
 }
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ void mul4(const float (&x)[4], const float (&y)[4], float (&out)[4]) {
+  const unsigned long long l = mul2(pk(x[0], x[1]), pk(y[0], y[1]));
+  const unsigned long long h = mul2(pk(x[2], x[3]), pk(y[2], y[3]));
+  upk(l, out[0], out[1]);
+  upk(h, out[2], out[3]);
+}
 __device__ __forceinline__ float dot4(const float (&x)[4], const float (&y)[4]) {
   float a, b;
   upk(fma2(pk(x[2], x[3]), pk(y[2], y[3]), fma2(pk(x[0], x[1]), pk(y[0], y[1]), 0ull)), a, b);
