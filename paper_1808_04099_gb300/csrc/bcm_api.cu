@@ -451,9 +451,12 @@ Layout plan(const bcm_grid_desc* d, int n_slots, const MgHost& mg, MgLayout* ml)
   L.phi = take(n * S); L.ub = take(nub * S);
   L.p = take(n * 8); L.b = take(n * 8);
   L.bid = take(n); L.near_ = take(d->n_cubes);
-  L.r = take(n * V); L.p0 = take(n * V); L.p1 = take(n * V); L.q = take(n * V);
+  // r, p0, p1, w1, s0, s1 also hold the Crank-Nicolson iteration's corrections, in the
+  // state's type
+  const size_t VS = S > V ? S : V;
+  L.r = take(n * VS); L.p0 = take(n * VS); L.p1 = take(n * VS); L.q = take(n * V);
   L.e = take(d->precision == BCM_PREC_F64 ? 0 : n * 4);  // FP32 inner iterate
-  L.w1 = take(n * V); L.s0 = take(n * V); L.s1 = take(n * V);
+  L.w1 = take(n * VS); L.s0 = take(n * VS); L.s1 = take(n * VS);
   // fused PCG: r, q, p on the six face planes of every cube, two parities
   const bool fused_ok = d->precision != BCM_PREC_F64 && d->cells_per_edge == 16;
   L.face = fused_ok ? take((size_t)2 * d->n_cubes * 6 * 3 * 16 * 16 * sizeof(float)) : 0;
