@@ -93,7 +93,6 @@ __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" 
 struct ResShape {
   int lb, lk;          // log2 of the cube edge B and of the slab depth KS
   int ipb;             // items of the fullest block
-  int nls;             // sims a block may hold cells of (capacity)
   int mq;              // quads per thread whose K p / h is in shared memory (the rest: q)
   int multi;           // some block holds cells of several sims
   int o_g, o_q, o_item, o_21, o_tab, o_sim, o_red;  // byte offsets in dynamic shared memory
@@ -1088,9 +1087,10 @@ struct ResPlan {
 inline size_t up16(size_t b) { return (b + 15) & ~(size_t)15; }
 
 // The launch shape of a grid, or false when its vectors do not fit on chip: the slab
-// depth and the number of blocks of least estimated cycles per iteration.  An exchange
-// takes about 1500 + 10 cycles per block (measured: 1.6k on 16 blocks, 2.4k on 64, 3.1k
-// on 152), a cell 1 cycle of an SM in FP32 and 8 in FP64, a ghost entry 0.5 and 1.
+// depth and the number of blocks of least estimated cycles per iteration.  An exchange is put
+// at 1500 + 10 cycles per block (1.7k on 16 blocks, 3.0k on 152; measured without the sums 2.2k
+// and 3.1k, see above), a cell at 1 cycle of an SM in FP32 and 8 in FP64, a ghost entry at 0.5
+// and 1.
 template <class TV>
 bool res_shape(const Ctx& x, int nsm, size_t smem_max, ResPlan* out) {
   const int B = x.B, lb = B == 16 ? 4 : B == 8 ? 3 : 2;
