@@ -39,7 +39,7 @@ from paper_1808_04099_gb300 import workloads as W  # noqa: E402
 
 RTOL = 1e-8
 METRIC = "cell-updates/s per step & % HBM roofline, FP32+refine vs FP64 at residual 1e-8"
-FP64_INST_PER_CELL_ITER = 22.5  # FP64 instructions per cell of one FP64 PCG iteration (ncu)
+FP64_INST_PER_CELL_ITER = 20.5  # FP64 instructions per cell of a two-launch FP64 PCG iteration (ncu)
 
 # Algorithmic bytes per cell of each kernel class (halo reads of neighbour cubes are
 # counted 0: they are served by L2).  S = state/vector size (4 mixed, 8 FP64).
@@ -73,7 +73,8 @@ def bytes_per_cell(kernel: str, f64: bool, phi_frac: float) -> float:
 # += alpha p of the previous iteration rides on the staging of p; pass B r, q in, r
 # out), fused single-barrier (x, r, p in and out, q recomputed, plus the six face
 # planes of r, q, p written to the face array: 0.375 of a cell's values each for 16^3
-# cubes), the other forms two passes (pass A r, p in, p, q out; pass B x, p, r, q in,
+# cubes), on chip (x in and out where it is not in registers, the face planes of z out
+# and in), the other forms two passes (pass A r, p in, p, q out; pass B x, p, r, q in,
 # x, r out).
 def pcg_schedule_bytes(form: int, f64: bool) -> float:
     S = 8 if f64 else 4
@@ -87,6 +88,9 @@ PCG_SOURCES = ["bcm_pcg.cu", "bcm_persist.cuh", "bcm_cube.cuh", "bcm_internal.cu
 
 # ncu summary and the sources it was taken at, per persistent PCG form
 PROFILES = {1: (PROFILE, PCG_SOURCES),
+            3: ("profiles/pcg_onchip_sphere_16x8x8_B16_mixed.md",
+                ["bcm_pcg_res.cuh", "bcm_pcg_res32.cu", "bcm_quad.cuh", "bcm_persist.cuh",
+                 "bcm_cube.cuh", "bcm_internal.cuh", "bcm_kernels.h"]),
             5: ("profiles/pcg_fused_sphere_16x8x8_B16_mixed.md",
                 ["bcm_pcg_fused.cu", "bcm_bulk.cuh", "bcm_persist.cuh", "bcm_cube.cuh",
                  "bcm_internal.cuh", "bcm_kernels.h"])}
@@ -777,14 +781,12 @@ def gpu_arm(args, ws, rank, local):
             legs["adjoint_33M_fp64"] = leg_adjoint(dev, args, ws)
     # the FP64 PCG's bound: min(HBM, FP64 pipe).  The pipe issues one FP64 instruction
     # per lane whether it adds, multiplies or fuses, so its rate is the measured FMA
-    # rate over 2; the two-launch iteration executes 22.5 FP64 instructions per cell
-    # (pass A 16.8, pass B 5.7; ncu on 16^3 cubes,
+    # rate over 2; the two-launch iteration (this grid does not fit on chip in FP64)
+    # executes 20.5 FP64 instructions per cell (pass A 14.8, pass B 5.7; ncu on 16^3 cubes,
     # profiles/fp64_instructions_sphere_16x8x8_B8.md) against 6 x 8 bytes
     fp64_bound = None
     t_iter = None
-    if "pcg" in k64 and k64["pcg"].get("us_per_iter"):
-        t_iter = k64["pcg"]["us_per_iter"] * 1e-6
-    elif "cg_a" in k64 and "cg_b" in k64 and iters64:
+    if "cg_a" in k64 and "cg_b" in k64 and iters64:
         t_iter = (k64["cg_a"]["total_ms"] + k64["cg_b"]["total_ms"]) * 1e-3 / iters64
     if "fma_peak" in legs and t_iter:
         inst_cell = FP64_INST_PER_CELL_ITER

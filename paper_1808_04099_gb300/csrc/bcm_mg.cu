@@ -28,10 +28,10 @@
 //
 // What bounds it: the finest level moves 49 bytes a cell and iteration in FP32 (pass A 16,
 // down with pass B 24.5, up 8.5; 60 before, when x = S r was stored and read).  On 83M cells
-// (two levels) the three launches take 281, 405 and 277 us, 4.7, 5.0 and 2.5 TB/s (427, 470
-// and 410 us with padded tiles); on 4.2M cells 19.5, 25 and 19 us (31, 31, 39).  In FP64
-// they are bound by the FP64 pipe: 96, 131 and 122 us (138, 192, 151).  Below the finest
-// level it is latency: 5 launches, 58 us serialised at 1024 cubes, where there were 9 in 80.
+// (two levels) the three launches take 282, 416 and 280 us, 4.7, 4.9 and 2.5 TB/s (427, 470
+// and 410 us with padded tiles); on 4.2M cells 20, 26 and 19 us (31, 31, 39).  In FP64
+// they are bound by the FP64 pipe: 122, 160 and 144 us (138, 192, 151).  Below the finest
+// level it is latency: 7 launches, 63 us serialised at 1024 cubes, where there were 9 in 80.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -1032,8 +1032,8 @@ static cudaError_t up_quad_t(const Ctx& x, int l, const SolveParams& prm, int mo
 // First level of the coarse kernel: at most 4^3 cells per cube, and at most kCoarseCells cells
 // (a launch over all SMs does more of them faster).  A block takes kCoarseBlock cells, up to
 // the largest cluster: one SM does 1.7 FP64 operations a clock, so with 1024 cells a block
-// these levels took longer than the launches they replaced.  FP64 steps in us with a launch
-// per level, with 16k cells and 1024 a block, and with these: 128 cubes of 4^3 2031, 2312,
+// these levels took longer than the launches they replaced.  FP64 steps in us (before the
+// 8^3 tiles took two planes a thread) with a launch per level, with 16k cells and 1024 a block, and with these: 128 cubes of 4^3 2031, 2312,
 // 1868; 1728 of 4^3 3408, 3485, 3128; 16 of 8^3 2577, 2998, 2556; 128 of 8^3 3341, 3592,
 // 3084; 1024 of 16^3 31.4, 24.9, 24.3 ms.  2048 and 1024 cells, 256 and 64 a block: the same
 // within 2 %.

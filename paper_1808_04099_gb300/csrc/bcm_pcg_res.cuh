@@ -13,8 +13,8 @@
 // all cells left a smooth error in the pressure that later iterations do not see (relative
 // error at rtol 1e-12 on 246k cells 5.2e-13, now 1.6e-13; streaming form 1.4e-13).
 // A cell's neighbours in other items are six ghost planes per item in shared memory, which
-// hold the neighbours' p and are
-// advanced by the same recurrence p = z + beta p as the cells themselves, so the only
+// hold the neighbours' p and are advanced by the same recurrence p = z + beta p as the cells
+// themselves, so the only
 // values that cross between blocks are the z of the items' face cells (fz, one plane per
 // face, in L2).  An iteration is
 //   pass A  p = z + beta p on the cells and the ghost planes; K p; <p, Kp>
@@ -30,14 +30,13 @@
 // barrier_timeout_ns (BCM_E_TIMEOUT).
 //
 // What bounds it: the two exchanges on small grids (2.2k cycles among 16 blocks, 3.1k
-// among 152, with the sums 3-4k each); the FP64 pipe in FP64 (about 12 FP64 operations a
-// cell and iteration against the 22.5 of the two-launch form, which scales and recomputes
-// halo cells; 1.7 operations a cycle and SM); instruction latency at 16 warps per SM on
-// the largest FP32 grids.  Microseconds per iteration, two-launch (FP64) or streaming
-// (FP32) form before and this form now:
-//   FP64  8k cells (16 cubes of 8^3) 27.2 -> 9.8; 64^3 48.8 -> 16.9; 524k (8^3) 50.1 -> 23.5
-//   FP32  262k 14.5 -> 9.9; 524k (8^3) 16.0 -> 10.3; 24 sims, 312k cells 31.3 -> 16.8;
-//         4.2M 33.5 -> 28.7
+// among 152, with the sums 3-4k each); the FP64 pipe in FP64 (about 16 FP64 operations a
+// cell and iteration, 20 counted on 64^3 with the ghost planes of its thin slabs; 1.7 a cycle
+// and SM); instruction latency at 16 warps per SM on the largest FP32 grids.  Microseconds
+// per iteration in two launches (FP64) or streaming (FP32), and here:
+//   FP64  8k cells (16 cubes of 8^3) 28.8, 10.0; 64^3 48.2, 19.1; 524k (8^3) 47.9, 27.6
+//   FP32  262k 13.0, 8.3; 524k (8^3) 15.1, 9.5; 24 sims, 312k cells 33.5, 10.4; 4.2M 32.5,
+//         28.9
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>

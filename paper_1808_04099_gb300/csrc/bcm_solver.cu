@@ -179,9 +179,10 @@ __global__ __launch_bounds__(NT) void k_residual(DevGrid g, const double* __rest
 }
 
 // The same on whole cubes of 16^3 or 8^3 by quad tiles (bcm_quad.cuh).  It is bound by the
-// FP64 pipe: about 10 operations a cell in the mixed mode against 22 of the padded-tile
-// kernel (the neighbour sum six instead of eleven, ||rhs|| only in a solve's first cycle,
-// each thread's FP32 sums and diagonals in FP32): 4.2M cells in 180 us before, 128 us now.
+// FP64 pipe: about 14 operations a cell in the mixed mode against 22 of the padded-tile
+// kernel (differences along x and z shared by two cells, ||rhs|| only in a solve's first
+// cycle, each thread's FP32 sums and diagonals in FP32): 4.2M cells in 180 us before, 150 us
+// now.
 template <int B, class TV, bool MIXED>
 __global__ __launch_bounds__(QT<B, double>::NT, QT<B, double>::blocks) void k_residual_quad(
     DevGrid g, const double* __restrict__ b, const double* __restrict__ x, TV* __restrict__ r,
