@@ -33,6 +33,7 @@
 
 #include "bcm_internal.cuh"
 #include "bcm_kernels.h"
+#include "bcm_persist.cuh"
 
 namespace bcm {
 
@@ -511,18 +512,12 @@ constexpr size_t wav_smem() { return sizeof(double) * B * B * (B + 1); }
 template <int B>
 size_t wav_dec_smem(uint32_t wcap) { return wav_smem<B>() + 4 * ((size_t)wcap + 3); }
 
-template <class K>
-cudaError_t wav_allow(K kern, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <int B, class T>
 cudaError_t compress_t(const Ctx& x, const void* field, double step, uint32_t* zc,
                        uint32_t* cube_nbits, uint32_t* cube_k, uint32_t* off, int* err) {
   const double inv = wav_inv(step);
   auto kf = std::isnan(inv) ? k_wav_forward<B, T, true> : k_wav_forward<B, T, false>;
-  cudaError_t e = wav_allow(kf, wav_smem<B>());
+  cudaError_t e = allow_dynamic_smem(kf, wav_smem<B>());
   if (e != cudaSuccess) return e;
   kf<<<x.g.n_cubes, B * B, wav_smem<B>(), x.stream>>>((const T*)field, step, inv, zc,
                                                       cube_nbits, cube_k, err);
@@ -537,7 +532,7 @@ cudaError_t decompress_t(const Ctx& x, void* field, const uint32_t* in, size_t w
   auto kd = std::isnan(wav_inv(step)) ? k_wav_decode<B, T, true> : k_wav_decode<B, T, false>;
   const uint32_t wcap = std::min<uint32_t>(max_payload, 48u * B * B * B / 32u);
   const size_t sm = wav_dec_smem<B>(wcap);
-  cudaError_t e = wav_allow(kd, sm);
+  cudaError_t e = allow_dynamic_smem(kd, sm);
   if (e != cudaSuccess) return e;
   kd<<<x.g.n_cubes, B * B, sm, x.stream>>>(in, off, words, wcap, step, (T*)field, err);
   return cudaGetLastError();
